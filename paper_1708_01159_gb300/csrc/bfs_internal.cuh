@@ -281,6 +281,40 @@ __device__ __forceinline__ uint32_t ld_nc_u32(const uint32_t* p) {
   return v;
 }
 
+// Predicated accesses (nothing is accessed when p is false). Written as one
+// predicated instruction each, so that several in a row are in flight
+// together: with an `if` around each, the compiler branches around them and
+// waits for one's result before it issues the next.
+__device__ __forceinline__ int32_t ld_if(bool p, const int32_t* a, int32_t otherwise) {
+  int32_t x = otherwise;
+  asm("{\n .reg .pred q;\n setp.ne.s32 q, %2, 0;\n @q ld.global.s32 %0, [%1];\n}\n"
+               : "+r"(x)
+               : "l"(a), "r"((int)p));
+  return x;
+}
+
+__device__ __forceinline__ uint32_t ld_volatile_if(bool p, const uint32_t* a, uint32_t otherwise) {
+  uint32_t x = otherwise;
+  asm volatile("{\n .reg .pred q;\n setp.ne.s32 q, %2, 0;\n @q ld.volatile.global.u32 %0, [%1];\n}\n"
+               : "+r"(x)
+               : "l"(a), "r"((int)p)
+               : "memory");
+  return x;
+}
+
+__device__ __forceinline__ uint32_t atom_or_if(bool p, uint32_t* a, uint32_t bits, uint32_t otherwise) {
+  uint32_t x = otherwise;
+  asm volatile("{\n .reg .pred q;\n setp.ne.s32 q, %3, 0;\n @q atom.global.or.b32 %0, [%1], %2;\n}\n"
+               : "+r"(x)
+               : "l"(a), "r"(bits), "r"((int)p)
+               : "memory");
+  return x;
+}
+
+__device__ __forceinline__ void prefetch_l2_if(bool p, const void* a) {
+  asm volatile("{\n .reg .pred q;\n setp.ne.s32 q, %1, 0;\n @q prefetch.global.L2 [%0];\n}\n" ::"l"(a), "r"((int)p));
+}
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }

@@ -138,7 +138,11 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 // claims (atomicOr) issued, then the winners' row extents read, so the K
 // edges' memory round trips overlap instead of forming one dependent chain per
 // edge. The one thread whose atomicOr flips a vertex's bit writes its depth,
-// counts its out-degree and stages it.
+// counts its out-degree and stages it. Bound by these round trips; written as
+// predicated accesses because an `if` per edge made the compiler wait for each
+// claim and each row extent in turn (vertex push on R-MAT 14: 2.49 ms a
+// traversal with the branches, 1.85 ms without; virtual warps on its level of
+// 345k edges 78 -> 59 us; ER 2^21, level of 1.6M edges, 48 -> 41 us).
 // valid: bit k set when v[k] is an edge to visit.
 template <int K, int kCount = CM_BLOCK>
 __device__ __forceinline__ void visit_km(const DevGraph& g, const Level& lv, const Stage& s, const int32_t (&v)[K],
@@ -146,24 +150,25 @@ __device__ __forceinline__ void visit_km(const DevGraph& g, const Level& lv, con
   const bool filter = !lv.latency_bound;
   uint32_t word[K];
 #pragma unroll
-  for (int k = 0; k < K; ++k)
-    word[k] = (valid >> k) & 1u ? (filter ? ld_volatile_u32(lv.vis + (v[k] >> 5)) : 0u) : 0xffffffffu;
+  for (int k = 0; k < K; ++k) word[k] = ld_volatile_if(filter && ((valid >> k) & 1u), lv.vis + (v[k] >> 5), 0u);
   bool won[K];
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     const uint32_t bit = 1u << (v[k] & 31);
-    won[k] = false;
-    if (((valid >> k) & 1u) && !(word[k] & bit)) won[k] = (atomicOr(lv.vis + (v[k] >> 5), bit) & bit) == 0u;
+    word[k] = atom_or_if(((valid >> k) & 1u) && !(word[k] & bit), lv.vis + (v[k] >> 5), bit, bit);
   }
-  int32_t d[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) won[k] = !((word[k] >> (v[k] & 31)) & 1u);
+  int32_t b0[K], d[K];
 #pragma unroll
   for (int k = 0; k < K; ++k) {
-    d[k] = 0;
-    if (won[k]) {
-      const int32_t b0 = g.off[v[k]];
-      d[k] = g.off[v[k] + 1] - b0;
-      if (!filter && d[k] > 0) prefetch_l2(g.idx + b0);
-    }
+    b0[k] = ld_if(won[k], g.off + v[k], 0);
+    d[k] = ld_if(won[k], g.off + v[k] + 1, 0);
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    d[k] -= b0[k];
+    prefetch_l2_if(!filter && d[k] > 0, g.idx + b0[k]);
   }
 #pragma unroll
   for (int k = 0; k < K; ++k)
@@ -179,11 +184,21 @@ __device__ __forceinline__ void visit_km(const DevGraph& g, const Level& lv, con
     }
 }
 
-// The first nv entries of v are edges to visit.
+// The first nv entries of v are edges to visit, four in flight at a time (more
+// do not fit the registers a thread has at four blocks per SM).
 template <int K, int kCount = CM_BLOCK>
 __device__ __forceinline__ void visit_k(const DevGraph& g, const Level& lv, const Stage& s, const int32_t (&v)[K],
                                         int nv, unsigned long long& edges) {
-  visit_km<K, kCount>(g, lv, s, v, nv >= 32 ? 0xffffffffu : (1u << nv) - 1u, edges);
+  constexpr int kAtOnce = K < 4 ? K : 4;
+  static_assert(K % kAtOnce == 0, "whole groups");
+#pragma unroll
+  for (int k = 0; k < K; k += kAtOnce) {
+    int32_t w[kAtOnce];
+#pragma unroll
+    for (int j = 0; j < kAtOnce; ++j) w[j] = v[k + j];
+    const int left = min(max(nv - k, 0), kAtOnce);
+    visit_km<kAtOnce, kCount>(g, lv, s, w, (1u << left) - 1u, edges);
+  }
 }
 
 template <typename T>
