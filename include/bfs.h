@@ -149,7 +149,10 @@ typedef struct bfs_run_stats {
   int32_t levels;            /* nonempty levels (max depth + 1) */
   int32_t status;            /* device-side status word (BFS_OK or BFS_ERR_TIMEOUT) */
   /* Per-level log, optional (set pointers to NULL to skip). Entry L describes
-   * the frontier of level L and the variant that expanded it. At most
+   * the frontier of level L and the variant that expanded it (under the tree,
+   * the variant it chose: on a graph whose out-degrees are at most 8, the
+   * persistent and graph drivers expand a small level it gives to a push
+   * variant by that push on one thread-block cluster). At most
    * log_capacity entries are written; levels beyond it are counted only. */
   int32_t log_capacity;
   int32_t* log_variant;      /* host, log_capacity entries */
@@ -176,7 +179,9 @@ int bfs_version(void);
  * list is the out-neighbours of its vertex. The library copies both arrays into
  * device memory it owns (the caller keeps ownership of its buffers), computes
  * the out-degree statistics the decision tree uses (Section 4.1), and, without
- * BFS_SYMMETRIC, builds the transpose that the pull variant reads. Self-loops
+ * BFS_SYMMETRIC, builds the transpose that the pull variant reads. A graph whose
+ * out-degrees are at most 8 also gets a record of every vertex's neighbours (16
+ * or 32 bytes a vertex), if that fits the device. Self-loops
  * and duplicate entries are allowed and never change a depth. Synchronous.
  * The CSR is always validated (a malformed one would make kernels read out
  * of bounds). Errors: BFS_ERR_INVALID_ARG (n < 1, n or m >= 2^31, null

@@ -193,6 +193,7 @@ constexpr int kMaxWorkspaces = 64;
 
 struct Shapes {
   int init, push_thread, push_warp, push_cta, pe, pull, edge_list;
+  int cluster;  // blocks per cluster of the persistent kernel (1: none)
   int persist;  // cooperative grid of the persistent kernel (0: not supported)
   int profile;  // cooperative grid of the per-level timing kernel (the persistent grid when it fits)
 };
@@ -346,8 +347,17 @@ int build_graph(bfs_graph* g, Workspace* ws) {
   CU(cudaGraphAddNode(&wnode, ws->graph, &ws->start_node, nullptr, 1, &wp));
   cudaGraph_t body = wp.conditional.phGraph_out[0];
 
-  cudaGraphNode_t decide;
-  TRY(add_kernel(body, &decide, nullptr, reinterpret_cast<const void*>(&k_decide), 1, kDecideThreads, ka));
+  cudaGraphNode_t decide, small;
+  const bool has_small = g->shapes.cluster > 1;
+  if (has_small) {
+    TRY(add_kernel(body, &small, nullptr, small_levels_kernel(g->dg.rec_w), g->shapes.cluster, kThreads, ka));
+    cudaKernelNodeAttrValue cl{};
+    cl.clusterDim.x = (unsigned)g->shapes.cluster;
+    cl.clusterDim.y = cl.clusterDim.z = 1;
+    CU(cudaGraphKernelNodeSetAttribute(small, cudaKernelNodeAttributeClusterDimension, &cl));
+  }
+  TRY(add_kernel(body, &decide, has_small ? &small : nullptr, reinterpret_cast<const void*>(&k_decide), 1,
+                 kDecideThreads, ka));
 
   cudaGraphConditionalHandle hs;
   CU(cudaGraphConditionalHandleCreate(&hs, body, 0, 0));
@@ -725,8 +735,21 @@ int launch_persistent(bfs_graph* g, Workspace* ws, int32_t root, int32_t* depth,
   int32_t stall = take_stall();
   void* args[] = {&dg, &b, &st, &depth, &root, &forced, &tree, &nodes, &qs, &epoch, &stall};
   const int grid = grid_blocks > 0 ? std::min(grid_blocks, g->shapes.persist) : g->shapes.persist;
-  CU(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_bfs_persistent), dim3(grid), dim3(kThreads), args, 0,
-                                 stream));
+  int cluster = g->shapes.cluster;
+  while (cluster > 1 && grid % cluster) cluster /= 2;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)cluster;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kThreads);
+  cfg.stream = stream;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  CU(cudaLaunchKernelExC(&cfg, persistent_kernel(dg.rec_w), args));
   return BFS_OK;
 }
 
@@ -1335,7 +1358,28 @@ int bfs_graph_create(const int32_t* row_offsets, const int32_t* col_indices, int
     cleanup();
     return r;
   }
+  // vertex records where every list is short (k_records); a graph they do not
+  // fit beside is used without
+  int32_t* rec = nullptr;
+  const int32_t rec_w = g->stats6[4] <= 4 ? 4 : g->stats6[4] <= 8 ? 8 : 0;
+  if (rec_w > 0) {
+    if (cudaMalloc(&rec, (size_t)n * rec_w * 4) == cudaSuccess) {
+      g->allocs.push_back(rec);
+      g->bytes += (size_t)n * rec_w * 4;
+      k_records<<<blocks, kThreads>>>(off, idx, (int32_t)n, rec_w, rec);
+      e = cudaDeviceSynchronize();
+      if (e != cudaSuccess) {
+        cleanup();
+        return fail(BFS_ERR_CUDA, "vertex records: %s", cudaGetErrorString(e));
+      }
+    } else {
+      cudaGetLastError();
+      rec = nullptr;
+    }
+  }
   DevGraph& dg = g->dg;
+  dg.rec = rec;
+  dg.rec_w = rec ? rec_w : 0;
   dg.off = off;
   dg.idx = idx;
   dg.in_off = in_off;
@@ -1366,11 +1410,38 @@ int bfs_graph_create(const int32_t* row_offsets, const int32_t* col_indices, int
   // the persistent kernel needs every block resident: one full occupancy wave
   int coop = 0, per_sm = 0;
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, g->device);
-  if (coop && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, reinterpret_cast<const void*>(&k_bfs_persistent),
-                                                            kThreads, 0) == cudaSuccess && per_sm > 0)
+  void* const persistent = persistent_kernel(dg.rec_w);
+  if (coop && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persistent, kThreads, 0) == cudaSuccess &&
+      per_sm > 0)
     s.persist = g->sms * std::min(per_sm, 8);
   else
     s.persist = 0;
+  // Graphs with vertex records run their small levels on one cluster, so their
+  // grid is launched in clusters. Clusters of 16 blocks leave 80 of the 608
+  // blocks of a GB300 out (8: 16 of them); a 4096^2 grid traversal takes 17 ms
+  // with 16 and 32 ms with 8, where the levels above half the queues' size go
+  // back to the whole grid.
+  s.cluster = 1;
+  if (s.persist > 0 && dg.rec_w > 0) {
+    const int want = kMaxCluster;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)want;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(want);
+    cfg.blockDim = dim3(kThreads);
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaFuncSetAttribute(persistent, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaFuncSetAttribute(small_levels_kernel(dg.rec_w), cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+            cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&clusters, persistent, &cfg) == cudaSuccess && clusters > 0) {
+      s.cluster = want;
+      s.persist = std::min(s.persist / want, clusters) * want;
+    }
+  }
   per_sm = 0;
   if (s.persist > 0 && cudaOccupancyMaxActiveBlocksPerMultiprocessor(
                            &per_sm, reinterpret_cast<const void*>(&k_profile_level), kThreads, 0) == cudaSuccess)

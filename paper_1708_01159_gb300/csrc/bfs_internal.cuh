@@ -162,6 +162,10 @@ struct DevGraph {
   // tests it first, since a high-degree in-neighbour is the likeliest to be
   // in an early frontier
   const int32_t* hint;
+  // vertex records, or null: the rec_w (4 or 8) out-neighbours of every vertex,
+  // -1 past its degree; only for graphs of no larger out-degree
+  const int32_t* rec;
+  int32_t rec_w;
   int32_t n;
   int32_t m;
   int32_t words;  // ceil(n / 32)
@@ -169,6 +173,19 @@ struct DevGraph {
   int32_t n_active;  // vertices with at least one in- or out-edge (the others start visited)
   int32_t vw_policy;  // virtual-warp width policy of the push_warp variant (VW_*)
   long long gfeat[F_NUM];  // the graph features (is_graph_feature); level slots unused
+};
+
+// The traversal between two levels: level L's frontier has f vertices and e
+// edges, not yet counted in discovered and reached.
+struct TravState {
+  long long discovered, reached;
+  unsigned long long e;
+  unsigned int f;
+  int32_t L;
+  int32_t prev;        // variant of level L - 1
+  int32_t force_full;  // level L runs on the whole grid even if it is small
+  int32_t ok;
+  unsigned int exchanges;  // level-end messages so far (both mbarriers' phases follow from it)
 };
 
 struct RunState {
@@ -205,6 +222,12 @@ struct RunState {
   unsigned long long tail3[3];
   unsigned long long edg3[3];
   unsigned long long bar64;
+  // persistent driver, small levels: tail of the queue the leader leaves, the
+  // state it publishes, the runs published, its current level (a sign of life)
+  unsigned long long small_tail;
+  TravState small_out;
+  unsigned int small_seq;
+  int32_t small_beat;
   unsigned int run_epoch;       // persistent driver: epoch of the launch whose block 0 reset the barrier state
   int32_t pad3_;
   int32_t log_cap;
@@ -288,6 +311,15 @@ __device__ __forceinline__ uint32_t ld_nc_u32(const uint32_t* p) {
 __device__ __forceinline__ int32_t ld_if(bool p, const int32_t* a, int32_t otherwise) {
   int32_t x = otherwise;
   asm("{\n .reg .pred q;\n setp.ne.s32 q, %2, 0;\n @q ld.global.s32 %0, [%1];\n}\n"
+               : "+r"(x)
+               : "l"(a), "r"((int)p));
+  return x;
+}
+
+// The same, issued where it stands (the compiler moves the one above to its use).
+__device__ __forceinline__ int32_t ld_now_if(bool p, const int32_t* a, int32_t otherwise) {
+  int32_t x = otherwise;
+  asm volatile("{\n .reg .pred q;\n setp.ne.s32 q, %2, 0;\n @q ld.global.s32 %0, [%1];\n}\n"
                : "+r"(x)
                : "l"(a), "r"((int)p));
   return x;

@@ -347,30 +347,31 @@ __device__ __forceinline__ int32_t qs_eval_warp(const QsTree& q, int32_t L, long
 // lane 2k + 1: upper bound; k = frontier, discovered, frontier edges, level).
 __device__ __forceinline__ bool in_leaf_box(int32_t bound, int32_t L, long long f, long long e, long long discovered) {
   const uint32_t lane = lane_id();
-  const long long x = lane < 2 ? f : lane < 4 ? discovered : lane < 6 ? e : (long long)L;
-  const bool ok = (lane & 1u) ? x <= (long long)bound : x >= (long long)bound;
+  // every level feature lies in [0, 2^31)
+  const int32_t x = lane < 2 ? (int32_t)f : lane < 4 ? (int32_t)discovered : lane < 6 ? (int32_t)e : L;
+  const bool ok = (lane & 1u) ? x <= bound : x >= bound;
   return __all_sync(kFull, lane >= 8u || ok);
 }
 
-// Section 4.1 unknown-prediction rule on a walk's result (or the forced
-// variant), and the virtual-warp width under the graph's policy: the rule is
-// the power of two nearest above the frontier's mean degree floor(e / f),
-// clamped to [4, 32] (floor(e / f) <= k is e < (k + 1) f).
-__device__ __forceinline__ int32_t finish_variant(int32_t v, int32_t L, int32_t prev, long long f, long long e,
-                                                  int32_t* vw, bool forced, int32_t policy) {
-  if (!forced) {
-    if (v < 0 || v >= V_NUM) v = (L == 0) ? kLevel0Default : prev;  // unknown prediction
-    if (v < 0 || v >= V_NUM) v = kLevel0Default;
-  }
-  const int32_t rule = (f <= 0 || e < 5 * f) ? 4 : e < 9 * f ? 8 : e < 17 * f ? 16 : 32;
-  *vw = policy == VW_RULE_X2     ? min(32, 2 * rule)
-        : policy == VW_RULE_HALF ? max(4, rule / 2)
-        : policy == VW_4         ? 4
-        : policy == VW_8         ? 8
-        : policy == VW_16        ? 16
-        : policy == VW_32        ? 32
-                                 : rule;
+// Section 4.1 unknown-prediction rule on a walk's result.
+__device__ __forceinline__ int32_t known_variant(int32_t v, int32_t L, int32_t prev) {
+  if (v < 0 || v >= V_NUM) v = (L == 0) ? kLevel0Default : prev;  // unknown prediction
+  if (v < 0 || v >= V_NUM) v = kLevel0Default;
   return v;
+}
+
+// The virtual-warp width under the graph's policy: the rule is the power of
+// two nearest above the frontier's mean degree floor(e / f), clamped to [4,
+// 32] (floor(e / f) <= k is e < (k + 1) f).
+__device__ __forceinline__ int32_t warp_width(long long f, long long e, int32_t policy) {
+  const int32_t rule = (f <= 0 || e < 5 * f) ? 4 : e < 9 * f ? 8 : e < 17 * f ? 16 : 32;
+  return policy == VW_RULE_X2     ? min(32, 2 * rule)
+         : policy == VW_RULE_HALF ? max(4, rule / 2)
+         : policy == VW_4         ? 4
+         : policy == VW_8         ? 8
+         : policy == VW_16        ? 16
+         : policy == VW_32        ? 32
+                                  : rule;
 }
 
 // ---------------------------------------------------------------------------
@@ -1128,6 +1129,7 @@ __global__ void __launch_bounds__(kThreads) k_init(DevGraph g, Buffers b, RunSta
     st->frontier_edges = 0;
     st->discovered = 0;
     st->edges_reached = 0;
+    st->small_tail = 0;
     // the root is the output of "level -1": the first decide turns it into the frontier of level 0
     b.q[1][0] = root;
     st->next_count = 1;
@@ -1196,8 +1198,8 @@ __global__ void __launch_bounds__(kDecideThreads) k_decide(DevGraph g, Buffers b
   if (threadIdx.x != 0) return;
   if (v < 0 && qs == nullptr && s.tree != nullptr && s.tree_nodes > 0)
     v = walk_tree(g, s.tree, s.tree_nodes, L, f, e, discovered);
-  int32_t vw = 32;
-  v = finish_variant(v, L, s.variant, f, e, &vw, s.forced >= 0, s.vw_policy);
+  if (s.forced < 0) v = known_variant(v, L, s.variant);
+  const int32_t vw = warp_width(f, e, s.vw_policy);
   for (int i = 0; i < F_NUM; ++i) s.feat[i] = feature_value(g, i, L, f, e, discovered);
   s.variant = v;
   s.vw = vw;
@@ -1361,17 +1363,18 @@ static_assert(2 * kCtaChunk <= 2 * kPeSlot, "union sizing");
 static_assert(pull_scratch_ints<kPullWordsPersistent>() <= 2 * kPeSlot, "union sizing");
 
 // Level L of a persistent traversal (frontier in q[L & 1], appending to
-// q[(L + 1) & 1] and to the (L + 1) % 3 level words; current bitmap vis[vsel]).
+// q[(L + 1) & 1] and to the level words of the given slot; current bitmap
+// vis[vsel]).
 __device__ __forceinline__ Level persistent_level(const DevGraph& g, const Buffers& b, RunState* st, int32_t* depth,
                                                   int32_t L, unsigned int f, unsigned long long e,
-                                                  long long discovered, uint32_t vsel) {
+                                                  long long discovered, uint32_t vsel, uint32_t slot) {
   Level lv;
   lv.qin = (L & 1) ? b.q[1] : b.q[0];
   lv.qout = (L & 1) ? b.q[0] : b.q[1];
   lv.vis = vsel ? b.vis[1] : b.vis[0];
   lv.vis_next = vsel ? b.vis[0] : b.vis[1];
   lv.depth = depth;
-  lv.tail = &st->tail3[(L + 1) % 3];
+  lv.tail = &st->tail3[slot];
   lv.next_depth = L + 1;
   lv.frontier = (int32_t)f;
   lv.latency_bound = (long long)e < kLatencyEdges;
@@ -1414,16 +1417,74 @@ __device__ __forceinline__ unsigned long long persistent_level_work(const DevGra
   return block_sum_u64(edges);
 }
 
+// The tree's choice of a level's variant, for every lane of the calling warp.
+struct TreeChoice {
+  const QsTree* qs;  // bit-parallel form (shared memory), or null
+  const TreeNode* tree;
+  int32_t nodes;
+  // lanes 0-7 of each warp: the box of the leaf the last evaluated level
+  // reached (in_leaf_box); leaf < 0 until a level has been evaluated
+  mutable int32_t bound, leaf;
+
+  // Section 4.1's rule for unknown predictions included.
+  __device__ __forceinline__ int32_t choose(const DevGraph& g, int32_t L, unsigned int f, long long e,
+                                            long long discovered, int32_t prev) const {
+    int32_t v = -1;
+    if (qs != nullptr) {
+      // same leaf box as the previous level: the walk reaches the same leaf, and
+      // the level repeats the previous level's choice (for an unknown leaf too)
+      if (leaf >= 0 && in_leaf_box(bound, L, f, e, discovered)) {
+        v = prev;
+      } else {
+        leaf = qs_leaf_warp(*qs, L, f, e, discovered);
+        v = leaf >= 0 ? qs->leaf[leaf] : -1;
+        bound = (leaf >= 0 && lane_id() < 8u) ? qs->box[leaf][lane_id()] : 0;
+      }
+    } else if (tree != nullptr && nodes > 0) {
+      v = walk_tree(g, tree, nodes, L, f, e, discovered);
+    }
+    return known_variant(v, L, prev);
+  }
+};
+
+// The per-level log's buffers, read once per launch.
+struct RunLog {
+  int32_t cap;
+  int32_t* variant;
+  long long* frontier;
+  long long* edges;
+  long long* time;
+};
+
+__device__ __forceinline__ void log_level(const RunLog& log, int32_t L, int32_t v, unsigned int f, long long e) {
+  if (L < log.cap) {
+    log.variant[L] = v;
+    log.frontier[L] = f;
+    log.edges[L] = e;
+    log.time[L] = (long long)global_ns();
+  }
+}
+
+}  // namespace bfs
+
+#include "bfs_small.cuh"
+
+namespace bfs {
+
 // epoch: a number the host changes on every launch on this workspace. Block 0
 // clears the barrier counter and the status word left by the previous run
 // (which a failed run may leave set) and then publishes epoch; every other
 // block waits for it before its first barrier, so no separate reset launch is
 // needed.
 // stall: STALL_NONE, or the test hook's choice of one bounded wait to run out.
-__global__ void __launch_bounds__(kThreads, 4) k_bfs_persistent(DevGraph g, Buffers b, RunState* st, int32_t* depth,
-                                                             int32_t root, int32_t forced, const TreeNode* tree,
-                                                             int32_t tree_nodes, const QsTree* qs, uint32_t epoch,
-                                                             int32_t stall) {
+// kRecord: 0, or the entries of the graph's vertex records (4 or 8); then small
+// levels run on the leader cluster (bfs_small.cuh).
+template <int kRecord>
+__global__ void __launch_bounds__(kThreads, 4) k_bfs_persistent(const __grid_constant__ DevGraph g,
+                                                             const __grid_constant__ Buffers b, RunState* st,
+                                                             int32_t* depth, int32_t root, int32_t forced,
+                                                             const TreeNode* tree, int32_t tree_nodes,
+                                                             const QsTree* qs, uint32_t epoch, int32_t stall) {
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     st->t_entry = (long long)global_ns();
     st->bar64 = 0;
@@ -1432,11 +1493,17 @@ __global__ void __launch_bounds__(kThreads, 4) k_bfs_persistent(DevGraph g, Buff
       st->tail3[k] = 0;
       st->edg3[k] = 0;
     }
+    st->small_tail = 0;
+    st->small_seq = 0;
+    st->small_beat = 0;
     st_release_u32(&st->run_epoch, epoch);
   }
   __shared__ alignas(128) int32_t ubuf[2 * kPeSlot];
+  static_assert(2 * kPeSlot >= 4 * kCandCap && kStageCap >= kWonCap, "the leader's queues");
   __shared__ alignas(8) uint64_t bar[2];
   __shared__ int s_split[2];
+  __shared__ SmallShared s_small;
+  __shared__ RunLog s_log;
   // the tree is evaluated by every warp every level: its bit-parallel form
   // (trees of up to 64 leaves) is kept in shared memory; larger trees are
   // walked in global memory
@@ -1456,6 +1523,11 @@ __global__ void __launch_bounds__(kThreads, 4) k_bfs_persistent(DevGraph g, Buff
     st->forced = forced;
     b.q[0][0] = root;
   }
+  if (threadIdx.x == 0) {
+    s_log = RunLog{st->log_cap, st->log_variant, st->log_frontier, st->log_edges, st->log_time};
+    mbar_init(&s_small.bar[0], 1);
+    mbar_init(&s_small.bar[1], 1);
+  }
   cta_pipe_init(bar);
   CtaPipe pp{ubuf, bar, 0u, 0u, stall == STALL_BULK_COPY ? 16u : 0u};
   // the previous run's barrier state is cleared before any block arrives
@@ -1464,64 +1536,147 @@ __global__ void __launch_bounds__(kThreads, 4) k_bfs_persistent(DevGraph g, Buff
     while (ld_acquire_u32(&st->run_epoch) != epoch)
       if (global_ns() - t0 > kWaitLimitNs) break;  // the first barrier then times out and reports it
   }
-  int32_t L = 0;
-  long long discovered = 0, reached = 0;
-  int32_t prev = -1;
+  // small levels go to cluster 0 when the tree drives the run (a forced
+  // variant is timed as itself; a stalled launch keeps its barriers)
+  const bool small_on =
+      kRecord > 0 && forced < 0 && stall == STALL_NONE && cluster_size() > 1u && cluster_size() <= (uint32_t)kMaxCluster;
   uint32_t vsel = 0;
-  // lanes 0-7 of each warp: the box of the leaf the last evaluated level
-  // reached (in_leaf_box); box_leaf < 0 until a level has been evaluated
-  int32_t box_bound = 0, box_leaf = -1;
+  uint32_t slot = 0;  // level words: this level's slot (the levels run on the whole grid, modulo 3)
+  const TreeChoice tc{use_qs ? &s_qs : nullptr, tree, tree_nodes, 0, -1};
+  if (threadIdx.x == 0) {
+    s_small.out.reached = 0;
+    s_small.out.exchanges = 0;
+    s_small.runs = 0;
+  }
+  int32_t L = 0, prev = -1;
+  bool force_full = false;
+  long long discovered = 0;
   // level 0's frontier is the root; later levels' f and e arrive with the barrier
   unsigned int f = 1;
   unsigned long long e = (unsigned long long)(g.off[root + 1] - g.off[root]);
   unsigned long long bar_target = 0;  // this block's copy of the grid barriers' arrival target
   bool ok = grid_arrive_wait(&st->bar64, bar_target, &st->status, stall == STALL_GRID_BARRIER ? 1u : 0u);
-  for (; ok; ++L) {
-    discovered += f;
-    reached += (long long)e;
-    if (f == 0) break;
-    if (L > g.n || discovered > g.n) {  // corrupted state: stop with an error
+  while (ok && f != 0) {
+    if (L > g.n || discovered + f > g.n) {  // corrupted state: stop with an error
       if (blockIdx.x == 0 && threadIdx.x == 0) st->status = ST_TIMEOUT;
       break;
     }
-    int32_t vw = 32;
-    int32_t v = forced;
-    if (v < 0 && use_qs) {
-      // same leaf box as the previous level: the walk reaches the same leaf, and
-      // the level repeats the previous level's choice (for an unknown leaf too)
-      if (box_leaf >= 0 && in_leaf_box(box_bound, L, f, (long long)e, discovered)) {
-        v = prev;
+    const int32_t v = forced >= 0 ? forced : tc.choose(g, L, f, (long long)e, discovered + f, prev);
+    if (kRecord > 0 && small_on && !force_full && v != V_PULL && small_fits(e, cluster_size())) {
+      if (blockIdx.x < cluster_size()) {
+        if (threadIdx.x == 0) {
+          s_small.out.discovered = discovered;
+          s_small.out.e = e;
+          s_small.out.f = f;
+          s_small.out.L = L;
+          s_small.out.prev = prev;
+        }
+        __syncthreads();
+        small_run<kRecord == 8 ? 8 : 4>(g, b, vsel ? b.vis[1] : b.vis[0], depth, st, tc.qs, tree, tree_nodes, s_log, s_small, ubuf, stage.buf,
+                  v);
       } else {
-        box_leaf = qs_leaf_warp(s_qs, L, f, (long long)e, discovered);
-        v = box_leaf >= 0 ? s_qs.leaf[box_leaf] : -1;
-        box_bound = (box_leaf >= 0 && lane_id() < 8u) ? s_qs.box[box_leaf][lane_id()] : 0;
+        small_park(st, s_small);
       }
-    } else if (v < 0 && tree != nullptr && tree_nodes > 0)
-      v = walk_tree(g, tree, tree_nodes, L, f, (long long)e, discovered);
-    v = finish_variant(v, L, prev, f, (long long)e, &vw, forced >= 0, g.vw_policy);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      st->tail3[(L + 2) % 3] = 0;  // the slot of level L - 2's barrier, which every block has left
-      st->edg3[(L + 2) % 3] = 0;
-      if (L < st->log_cap) {
-        st->log_variant[L] = v;
-        st->log_frontier[L] = f;
-        st->log_edges[L] = (long long)e;
-        st->log_time[L] = (long long)global_ns();
-      }
+      __syncthreads();
+      discovered = s_small.out.discovered;
+      e = s_small.out.e;
+      f = s_small.out.f;
+      L = s_small.out.L;
+      prev = s_small.out.prev;
+      force_full = s_small.out.force_full != 0;
+      ok = s_small.out.ok != 0;
+      tc.leaf = -1;  // prev is not the class of this block's last leaf any more
+      __syncthreads();
+      continue;
     }
-    const Level lv = persistent_level(g, b, st, depth, L, f, e, discovered, vsel);
+    force_full = false;
+    discovered += f;
+    if (threadIdx.x == 0) s_small.out.reached += (long long)e;
+    const uint32_t next = slot == 2u ? 0u : slot + 1u;
+    if (blockIdx.x == 0) {
+      if (threadIdx.x == 0) {
+        const uint32_t after = next == 2u ? 0u : next + 1u;
+        st->tail3[after] = 0;  // the slot of a barrier every block has left
+        st->edg3[after] = 0;
+      }
+      if (threadIdx.x == kThreads - 1) log_level(s_log, L, v, f, (long long)e);
+    }
+    const Level lv = persistent_level(g, b, st, depth, L, f, e, discovered, vsel, next);
+    const int32_t vw = warp_width(f, (long long)e, g.vw_policy);
     const unsigned long long e_block = persistent_level_work(g, b, st, lv, v, vw, stage, pp, ubuf, s_split, bar_target);
     if (v == V_PULL) vsel ^= 1u;
     prev = v;
-    ok = level_arrive_wait(&st->tail3[(L + 1) % 3], &st->edg3[(L + 1) % 3], e_block, &st->status, &f, &e,
+    ok = level_arrive_wait(&st->tail3[next], &st->edg3[next], e_block, &st->status, &f, &e,
                            (stall == STALL_LEVEL_BARRIER && L == 0) ? 1u : 0u);
+    slot = next;
+    ++L;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     st->levels = L;
-    if (L < st->log_cap) st->log_time[L] = (long long)global_ns();
+    if (L < s_log.cap) s_log.time[L] = (long long)global_ns();
     st->discovered = discovered;
-    st->edges_reached = reached;
+    st->edges_reached = s_small.out.reached;
   }
+  // no block of a cluster ends while another may still send to its shared memory
+  if (kRecord > 0 && cluster_size() > 1u) cluster_barrier();
+}
+
+// Graph driver, before each level's decision, for graphs with vertex records
+// (one cluster): runs the next level and those after it while they are small,
+// and leaves the state as k_decide expects it (the output queue of the level
+// before is in q[qsel ^ 1]). In this driver level L's queue is q[(L + 1) & 1].
+// (777 x 1021 grid, 1,338 levels, in this driver: 17 us a level with a decision
+// and a level kernel each, 1.6 us in runs; 22 -> 2.2 ms a traversal.)
+template <int kRecord>
+__global__ void __launch_bounds__(kThreads) k_small_levels(const __grid_constant__ DevGraph g, Buffers b,
+                                                           RunState* st) {
+  __shared__ alignas(128) int32_t ubuf[4 * kCandCap];
+  __shared__ int32_t sbuf[kWonCap];
+  __shared__ SmallShared s_small;
+  __shared__ RunLog s_log;
+  const int32_t L = st->level + 1;
+  const unsigned int f = (unsigned int)st->next_count;
+  const unsigned long long e = st->next_edges;
+  const long long discovered = st->discovered;
+  // k_decide switches to the bitmap a pull level wrote; this kernel runs first
+  const uint32_t vsel = st->vsel ^ (uint32_t)(st->level >= 0 && st->variant == V_PULL);
+  if (st->forced >= 0 || st->status != ST_OK || f == 0 || !small_fits(e, cluster_size())) return;  // uniform
+  const TreeChoice tc{st->tree_qs, st->tree, st->tree_nodes, 0, -1};
+  const int32_t v = tc.choose(g, L, f, (long long)e, discovered + f, st->variant);
+  if (v == V_PULL) return;  // uniform over the cluster: every block reads the same state
+  if (threadIdx.x == 0) {
+    s_log = RunLog{st->log_cap, st->log_variant, st->log_frontier, st->log_edges, st->log_time};
+    s_small.out = TravState{discovered, st->edges_reached, e, f, L, st->variant, 0, 1, 0u};
+    mbar_init(&s_small.bar[0], 1);
+    mbar_init(&s_small.bar[1], 1);
+    mbar_fence_init();
+  }
+  cluster_barrier();  // the state is read and every block's mbarriers are ready
+  const Buffers swapped{{b.q[1], b.q[0]}, {b.vis[0], b.vis[1]}, b.pe_scan, b.pe_beg, b.pe_bsum, b.pe_blocks_cap, 0};
+  small_run<kRecord>(g, swapped, vsel ? b.vis[1] : b.vis[0], st->depth, st, tc.qs, tc.tree, tc.nodes, s_log,
+                     s_small, ubuf, sbuf, v);
+  if (cluster_rank() == 0u && threadIdx.x == 0 && s_small.out.L > L) {
+    const TravState& t = s_small.out;
+    st->level = t.L - 1;
+    st->vsel = vsel;
+    st->qsel = (uint32_t)(t.L & 1);
+    st->variant = t.prev;
+    st->next_count = t.f;
+    st->next_edges = t.e;
+    st->discovered = t.discovered;
+    st->edges_reached = t.reached;
+  }
+  cluster_barrier();  // no block ends while another may still send to its shared memory
+}
+
+void* small_levels_kernel(int32_t record) {
+  return record == 8 ? reinterpret_cast<void*>(&k_small_levels<8>) : reinterpret_cast<void*>(&k_small_levels<4>);
+}
+
+void* persistent_kernel(int32_t record) {
+  return record == 8   ? reinterpret_cast<void*>(&k_bfs_persistent<8>)
+         : record == 4 ? reinterpret_cast<void*>(&k_bfs_persistent<4>)
+                       : reinterpret_cast<void*>(&k_bfs_persistent<0>);
 }
 
 // Per-level timing harness inside the persistent driver: one cooperative
@@ -1540,12 +1695,11 @@ __global__ void __launch_bounds__(kThreads, 4) k_profile_level(DevGraph g, Buffe
   BFS_DECLARE_STAGE(stage);
   cta_pipe_init(bar);
   CtaPipe pp{ubuf, bar, 0u, 0u, 0u};
-  int32_t vw = 32;
-  v = finish_variant(v, L, -1, f, (long long)e, &vw, true, g.vw_policy);
+  const int32_t vw = warp_width(f, (long long)e, g.vw_policy);
   unsigned long long bar_target = 0;
   if (!grid_arrive_wait(&st->bar64, bar_target, &st->status)) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) st->prof_t0 = (long long)global_ns();
-  const Level lv = persistent_level(g, b, st, depth, L, f, e, discovered, vsel);
+  const Level lv = persistent_level(g, b, st, depth, L, f, e, discovered, vsel, (uint32_t)((L + 1) % 3));
   const unsigned long long e_block = persistent_level_work(g, b, st, lv, v, vw, stage, pp, ubuf, s_split, bar_target);
   unsigned int fn = 0;
   unsigned long long en = 0;
@@ -1768,6 +1922,22 @@ __global__ void k_vis_init(const int32_t* off, const int32_t* in_off, int32_t n,
     if ((v & 31) == 0) {
       vis_init[v >> 5] = word;
       if (word) atomicAdd(isolated_count, (unsigned)__popc(word));
+    }
+  }
+}
+
+// Vertex records of a graph whose out-degrees are at most w (4 or 8).
+__global__ void k_records(const int32_t* off, const int32_t* idx, int32_t n, int32_t w, int32_t* rec) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
+    const int32_t b = off[v], d = off[v + 1] - b;
+    for (int32_t j = 0; j < w; j += 4) {
+      int4 r;
+      r.x = j < d ? idx[b + j] : -1;
+      r.y = j + 1 < d ? idx[b + j + 1] : -1;
+      r.z = j + 2 < d ? idx[b + j + 2] : -1;
+      r.w = j + 3 < d ? idx[b + j + 3] : -1;
+      *reinterpret_cast<int4*>(rec + v * w + j) = r;
     }
   }
 }

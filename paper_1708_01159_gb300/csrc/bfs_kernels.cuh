@@ -6,6 +6,7 @@
 namespace bfs {
 
 constexpr int kThreads = 256;     // block size of the level kernels
+constexpr int kMaxCluster = 16;   // blocks of a cluster that runs small levels (bfs_small.cuh)
 constexpr int kDecideThreads = 32;  // block size of k_decide: one warp evaluates the bit-parallel tree
 constexpr int kCtaChunk = 2048;   // int32 per shared-memory stage of the CTA variant (8 KB)
 constexpr int kCtaDirect = 512;   // adjacency shorter than this is read directly, not staged
@@ -31,9 +32,13 @@ __global__ void k_edge_list(DevGraph g, Buffers b, RunState* st);
 __global__ void k_rev_edge_list(DevGraph g, Buffers b, RunState* st);
 __global__ void k_build_origin(const int32_t* off, int32_t n, int32_t* origin);
 __global__ void k_undo_level(Buffers b, RunState* st);
-__global__ void k_bfs_persistent(DevGraph g, Buffers b, RunState* st, int32_t* depth, int32_t root, int32_t forced,
-                                 const TreeNode* tree, int32_t tree_nodes, const QsTree* qs, uint32_t epoch,
-                                 int32_t stall);
+// The persistent traversal kernel for graphs with vertex records of the given
+// width (0: none); parameters DevGraph, Buffers, RunState*, depth, root, forced,
+// tree, tree nodes, bit-parallel tree, epoch, stall.
+void* persistent_kernel(int32_t record);
+// The graph driver's kernel for runs of small levels (record 4 or 8; one cluster
+// of kThreads-thread blocks); parameters DevGraph, Buffers, RunState*.
+void* small_levels_kernel(int32_t record);
 __global__ void k_profile_level(DevGraph g, Buffers b, RunState* st, int32_t* depth, int32_t L, int32_t v, uint32_t f,
                                 unsigned long long e, long long discovered, uint32_t vsel);
 __global__ void k_profile_reset(RunState* st, int32_t slot);
@@ -52,6 +57,7 @@ __global__ void k_scan_reduce(const int32_t* in, int32_t len, long long* bsum);
 __global__ void k_scan_top(long long* bsum, int32_t nblocks);
 __global__ void k_scan_apply(const int32_t* in, int32_t len, const long long* bsum, int32_t* out);
 __global__ void k_tr_scatter(const int32_t* off, const int32_t* idx, int32_t n, int32_t* cursor, int32_t* in_idx);
+__global__ void k_records(const int32_t* off, const int32_t* idx, int32_t n, int32_t w, int32_t* rec);
 __global__ void k_pull_hint(const int32_t* off, const int32_t* in_off, const int32_t* in_idx, int32_t n,
                             int32_t* hint);
 __global__ void k_vis_init(const int32_t* off, const int32_t* in_off, int32_t n, int32_t words, uint32_t* vis_init,
