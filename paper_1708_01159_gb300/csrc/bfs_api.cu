@@ -192,7 +192,7 @@ struct Workspace {
 constexpr int kMaxWorkspaces = 64;
 
 struct Shapes {
-  int init, push_thread, push_warp, push_cta, pe, pull, edge_list;
+  int init, push_thread, push_warp, push_cta, push_edge, pull, edge_list;
   int cluster;  // blocks per cluster of the persistent kernel (1: none)
   int persist;  // cooperative grid of the persistent kernel (0: not supported)
   int profile;  // cooperative grid of the per-level timing kernel (the persistent grid when it fits)
@@ -370,17 +370,17 @@ int build_graph(bfs_graph* g, Workspace* ws) {
   CU(cudaGraphAddNode(&snode, body, &decide, nullptr, 1, &sp));
   cudaGraph_t* vb = sp.conditional.phGraph_out;
   const Shapes& s = g->shapes;
-  cudaGraphNode_t n0, n1, n2, n3;
+  cudaGraphNode_t n0, n1;
   TRY(add_kernel(vb[V_PUSH_THREAD], &n0, nullptr, reinterpret_cast<const void*>(&k_push_thread), s.push_thread,
                  kThreads, ka));
   TRY(add_kernel(vb[V_PUSH_WARP], &n0, nullptr, reinterpret_cast<const void*>(&k_push_warp), s.push_warp, kThreads,
                  ka));
   TRY(add_kernel(vb[V_PUSH_CTA], &n0, nullptr, reinterpret_cast<const void*>(&k_push_cta), s.push_cta, kThreads,
                  ka));
-  TRY(add_kernel(vb[V_PUSH_EDGE], &n0, nullptr, reinterpret_cast<const void*>(&k_pe_reduce), s.pe, kThreads, ka));
-  TRY(add_kernel(vb[V_PUSH_EDGE], &n1, &n0, reinterpret_cast<const void*>(&k_pe_top), 1, kThreads, ka));
-  TRY(add_kernel(vb[V_PUSH_EDGE], &n2, &n1, reinterpret_cast<const void*>(&k_pe_scan), s.pe, kThreads, ka));
-  TRY(add_kernel(vb[V_PUSH_EDGE], &n3, &n2, reinterpret_cast<const void*>(&k_pe_expand), s.pe, kThreads, ka));
+  TRY(add_kernel(vb[V_PUSH_EDGE], &n0, nullptr, reinterpret_cast<const void*>(&k_push_edge), s.push_edge, kThreads,
+                 ka));
+  if (g->dg.gfeat[F_DEG_MAX] >= kHeavy)
+    TRY(add_kernel(vb[V_PUSH_EDGE], &n1, &n0, reinterpret_cast<const void*>(&k_push_heavy), s.push_edge, kThreads, ka));
   TRY(add_kernel(vb[V_PULL], &n0, nullptr, reinterpret_cast<const void*>(&k_pull), s.pull, kThreads, ka));
   TRY(add_kernel(vb[V_EDGE_LIST], &n0, nullptr, reinterpret_cast<const void*>(&k_edge_list), s.edge_list, kThreads,
                  ka));
@@ -395,7 +395,6 @@ int create_workspace(bfs_graph* g, Workspace** out) {
   auto* ws = new Workspace;
   const int64_t n = g->dg.n;
   const int64_t words = g->dg.words;
-  const int64_t pe_blocks = (n + kPeTile - 1) / kPeTile + 2;
   int r = BFS_OK;
   void* p;
   auto A = [&](size_t bytes) -> void* {
@@ -407,10 +406,8 @@ int create_workspace(bfs_graph* g, Workspace** out) {
   ws->b.q[1] = static_cast<int32_t*>(A(n * 4));
   ws->b.vis[0] = static_cast<uint32_t*>(A(words * 4));
   ws->b.vis[1] = static_cast<uint32_t*>(A(words * 4));
-  ws->b.pe_scan = static_cast<int32_t*>(A((n + 1) * 4));
-  ws->b.pe_beg = static_cast<int32_t*>(A(n * 4));
-  ws->b.pe_bsum = static_cast<long long*>(A(pe_blocks * 8));
-  ws->b.pe_blocks_cap = (int32_t)pe_blocks;
+  ws->b.heavy_cap = (int32_t)std::min<int64_t>(n, kHeavyCap);
+  ws->b.heavy = static_cast<int32_t*>(A((size_t)ws->b.heavy_cap * 4));
   ws->st = static_cast<RunState*>(A(sizeof(RunState)));
   ws->log_cap = (int32_t)std::min<int64_t>(n + 1, 1 << 16);
   ws->log_variant = static_cast<int32_t*>(A(ws->log_cap * 4));
@@ -801,10 +798,8 @@ int launch_variant(bfs_graph* g, Workspace* ws, int v, cudaStream_t s, int32_t c
     case V_PUSH_WARP: k_push_warp<<<sh.push_warp, kThreads, 0, s>>>(dg, ws->b, ws->st); break;
     case V_PUSH_CTA: k_push_cta<<<sh.push_cta, kThreads, 0, s>>>(dg, ws->b, ws->st); break;
     case V_PUSH_EDGE:
-      k_pe_reduce<<<sh.pe, kThreads, 0, s>>>(dg, ws->b, ws->st);
-      k_pe_top<<<1, kThreads, 0, s>>>(dg, ws->b, ws->st);
-      k_pe_scan<<<sh.pe, kThreads, 0, s>>>(dg, ws->b, ws->st);
-      k_pe_expand<<<sh.pe, kThreads, 0, s>>>(dg, ws->b, ws->st);
+      k_push_edge<<<sh.push_edge, kThreads, 0, s>>>(dg, ws->b, ws->st);
+      if (dg.gfeat[F_DEG_MAX] >= kHeavy) k_push_heavy<<<sh.push_edge, kThreads, 0, s>>>(dg, ws->b, ws->st);
       break;
     case V_PULL: k_pull<<<sh.pull, kThreads, 0, s>>>(dg, ws->b, ws->st); break;
     case V_EDGE_LIST: k_edge_list<<<sh.edge_list, kThreads, 0, s>>>(dg, ws->b, ws->st); break;
@@ -878,10 +873,10 @@ int bfs::set_error_detail(int code, const char* msg) { return fail(code, "%s", m
 
 long long bfs::workspace_bytes(const bfs_graph* g) {
   const long long n = g->dg.n, words = g->dg.words;
-  // two queues, two bitmaps, edge-centric scan scratch, logs (a host-output
+  // two queues, two bitmaps, the edge-centric push's list, logs (a host-output
   // stage of 4 n bytes is added on a workspace's first host-output run)
-  return 4 * n * 2 + 4 * words * 2 + 4 * (n + 1) + 4 * n + 8 * ((n + kPeTile - 1) / kPeTile + 2) +
-         20 * std::min<long long>(n + 1, 1 << 16) + (long long)sizeof(RunState);
+  return 4 * n * 2 + 4 * words * 2 + 4 * std::min<long long>(n, kHeavyCap) +
+         28 * std::min<long long>(n + 1, 1 << 16) + (long long)sizeof(RunState);
 }
 
 int32_t bfs::graph_vertices(const bfs_graph* g) { return g->dg.n; }
@@ -1404,7 +1399,7 @@ int bfs_graph_create(const int32_t* row_offsets, const int32_t* col_indices, int
   s.push_thread = grid_for(reinterpret_cast<const void*>(&k_push_thread), g->sms, 8);
   s.push_warp = grid_for(reinterpret_cast<const void*>(&k_push_warp), g->sms, 8);
   s.push_cta = grid_for(reinterpret_cast<const void*>(&k_push_cta), g->sms, 8);
-  s.pe = grid_for(reinterpret_cast<const void*>(&k_pe_expand), g->sms, 8);
+  s.push_edge = grid_for(reinterpret_cast<const void*>(&k_push_edge), g->sms, 8);
   s.pull = grid_for(reinterpret_cast<const void*>(&k_pull), g->sms, 8);
   s.edge_list = grid_for(reinterpret_cast<const void*>(&k_edge_list), g->sms, 8);
   // the persistent kernel needs every block resident: one full occupancy wave

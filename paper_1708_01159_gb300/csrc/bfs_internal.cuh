@@ -9,7 +9,7 @@
 //   q[2][n]                     frontier queues (input / output, swapped per level)
 //   vis[2][ceil(n/32)]          visited bitmaps; push updates the current one in
 //                               place, pull reads the current and writes the other
-//   pe_*                        scratch of the edge-centric variant (degree scan)
+//   heavy                       vertices the edge-centric variant sets aside
 //   RunState                    level, counters, variant, status, log pointers
 #pragma once
 
@@ -221,6 +221,8 @@ struct RunState {
   // the high 24. bar64: monotonic arrival count of the other grid barriers.
   unsigned long long tail3[3];
   unsigned long long edg3[3];
+  unsigned int heavy3[3];  // vertices an edge-centric level set aside (graph and host-loop drivers: word 0)
+  int32_t pad5_;
   unsigned long long bar64;
   // persistent driver, small levels: tail of the queue the leader leaves, the
   // state it publishes, the runs published, its current level (a sign of life)
@@ -246,10 +248,8 @@ struct RunState {
 struct Buffers {
   int32_t* q[2];
   uint32_t* vis[2];
-  int32_t* pe_scan;      // exclusive scan of frontier degrees (f + 1 entries)
-  int32_t* pe_beg;       // off[u] of each frontier entry
-  long long* pe_bsum;    // per-block sums of the scan
-  int32_t pe_blocks_cap;
+  int32_t* heavy;        // vertices an edge-centric level sets aside
+  int32_t heavy_cap;
   int32_t pad_;
 };
 
@@ -325,13 +325,8 @@ __device__ __forceinline__ int32_t ld_now_if(bool p, const int32_t* a, int32_t o
   return x;
 }
 
-__device__ __forceinline__ uint32_t ld_volatile_if(bool p, const uint32_t* a, uint32_t otherwise) {
-  uint32_t x = otherwise;
-  asm volatile("{\n .reg .pred q;\n setp.ne.s32 q, %2, 0;\n @q ld.volatile.global.u32 %0, [%1];\n}\n"
-               : "+r"(x)
-               : "l"(a), "r"((int)p)
-               : "memory");
-  return x;
+__device__ __forceinline__ uint32_t ld_now_if(bool p, const uint32_t* a, uint32_t otherwise) {
+  return (uint32_t)ld_now_if(p, reinterpret_cast<const int32_t*>(a), (int32_t)otherwise);
 }
 
 __device__ __forceinline__ uint32_t atom_or_if(bool p, uint32_t* a, uint32_t bits, uint32_t otherwise) {

@@ -18,13 +18,11 @@
 // Section 3.1.4's first variant, a global atomic counter, with warp and block
 // aggregation in front of it), and adds the vertex's out-degree to the next
 // level's frontier-edge count.
-#include "bfs_kernels.cuh"
+#include "bfs_push.cuh"
 
 namespace bfs {
 
 namespace {
-
-constexpr unsigned kFull = 0xffffffffu;
 
 // ---- mbarrier + bulk async copy (TMA bulk, non-tensor) --------------------
 
@@ -70,36 +68,7 @@ __device__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity) {
   return true;
 }
 
-__device__ __forceinline__ uint32_t ld_volatile_u32(const uint32_t* p) {
-  return *reinterpret_cast<const volatile uint32_t*>(p);
-}
 
-
-// ---- output staging and per-edge visit --------------------------------------
-
-// No __restrict__ on the queue or bitmaps: inside the persistent kernel they are
-// rewritten every level, so they must not be read through the non-coherent
-// read-only cache.
-struct Level {
-  const int32_t* qin;
-  int32_t* qout;
-  uint32_t* vis;       // current visited bitmap (push updates it in place; pull reads it)
-  uint32_t* vis_next;  // the other bitmap (pull writes it)
-  int32_t* depth;
-  unsigned long long* tail;  // output queue tail (low 32 bits)
-  int32_t next_depth;
-  int32_t frontier;
-  int32_t latency_bound;  // the level's frontier has fewer than kLatencyEdges edges
-  int32_t pull_sparse;    // fewer than 1/16 of the vertices with edges are still unvisited
-};
-
-// Below this many frontier edges a level cannot fill the GPU: its time is the
-// latency of its chain of dependent memory accesses, not bandwidth. Such a
-// level claims targets without reading their bitmap word first (one round trip
-// less; the extra atomics cost nothing at this size) and prefetches the first
-// adjacency sector of every vertex it reaches into L2, so the next level's
-// list reads are L2 hits.
-constexpr long long kLatencyEdges = 1ll << 17;
 
 __device__ __forceinline__ Level load_level(const DevGraph& g, const Buffers& b, RunState* st) {
   Level lv;
@@ -114,121 +83,11 @@ __device__ __forceinline__ Level load_level(const DevGraph& g, const Buffers& b,
   lv.tail = &st->next_count;
   lv.next_depth = st->level + 1;
   lv.frontier = st->frontier;
+  lv.n_heavy = &st->heavy3[0];
+  lv.shared_scan = pe_shared(st->frontier, st->frontier_edges, g.gfeat[F_DEG_MAX] >= kHeavy);
   lv.latency_bound = st->frontier_edges < kLatencyEdges;
   lv.pull_sparse = (long long)g.n_active - st->discovered < (long long)(g.n_active >> 4);
   return lv;
-}
-
-// Newly reached vertices go through a block-local stage (see stage_put) into
-// the level's output queue.
-__device__ __forceinline__ void stage_push(const Stage& s, const Level& lv, int32_t v) {
-  stage_put(s, lv.qout, lv.tail, v);
-}
-
-__device__ __forceinline__ void stage_flush(const Stage& s, const Level& lv, unsigned int threshold) {
-  stage_drain(s, lv.qout, lv.tail, threshold);
-}
-
-__device__ __forceinline__ void prefetch_l2(const void* p) {
-  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
-
-// Top-down visit of up to K edges u -> v[k] (Section 3.1.2 push). The bitmap
-// words of all K targets are read (except on latency-bound levels), then the
-// claims (atomicOr) issued, then the winners' row extents read, so the K
-// edges' memory round trips overlap instead of forming one dependent chain per
-// edge. The one thread whose atomicOr flips a vertex's bit writes its depth,
-// counts its out-degree and stages it. Bound by these round trips; written as
-// predicated accesses because an `if` per edge made the compiler wait for each
-// claim and each row extent in turn (vertex push on R-MAT 14: 2.49 ms a
-// traversal with the branches, 1.85 ms without; virtual warps on its level of
-// 345k edges 78 -> 59 us; ER 2^21, level of 1.6M edges, 48 -> 41 us).
-// valid: bit k set when v[k] is an edge to visit.
-template <int K, int kCount = CM_BLOCK>
-__device__ __forceinline__ void visit_km(const DevGraph& g, const Level& lv, const Stage& s, const int32_t (&v)[K],
-                                         uint32_t valid, unsigned long long& edges) {
-  const bool filter = !lv.latency_bound;
-  uint32_t word[K];
-#pragma unroll
-  for (int k = 0; k < K; ++k) word[k] = ld_volatile_if(filter && ((valid >> k) & 1u), lv.vis + (v[k] >> 5), 0u);
-  bool won[K];
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const uint32_t bit = 1u << (v[k] & 31);
-    word[k] = atom_or_if(((valid >> k) & 1u) && !(word[k] & bit), lv.vis + (v[k] >> 5), bit, bit);
-  }
-#pragma unroll
-  for (int k = 0; k < K; ++k) won[k] = !((word[k] >> (v[k] & 31)) & 1u);
-  int32_t b0[K], d[K];
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    b0[k] = ld_if(won[k], g.off + v[k], 0);
-    d[k] = ld_if(won[k], g.off + v[k] + 1, 0);
-  }
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    d[k] -= b0[k];
-    prefetch_l2_if(!filter && d[k] > 0, g.idx + b0[k]);
-  }
-#pragma unroll
-  for (int k = 0; k < K; ++k)
-    if (won[k]) {
-      lv.depth[v[k]] = lv.next_depth;
-      edges += (unsigned long long)d[k];
-      if (kCount == CM_BLOCK)
-        stage_push(s, lv, v[k]);
-      else if (kCount == CM_WARP)
-        queue_append(lv.qout, lv.tail, v[k]);
-      else
-        lv.qout[(unsigned int)atomicAdd(lv.tail, 1ull)] = v[k];
-    }
-}
-
-// The first nv entries of v are edges to visit, four in flight at a time (more
-// do not fit the registers a thread has at four blocks per SM).
-template <int K, int kCount = CM_BLOCK>
-__device__ __forceinline__ void visit_k(const DevGraph& g, const Level& lv, const Stage& s, const int32_t (&v)[K],
-                                        int nv, unsigned long long& edges) {
-  constexpr int kAtOnce = K < 4 ? K : 4;
-  static_assert(K % kAtOnce == 0, "whole groups");
-#pragma unroll
-  for (int k = 0; k < K; k += kAtOnce) {
-    int32_t w[kAtOnce];
-#pragma unroll
-    for (int j = 0; j < kAtOnce; ++j) w[j] = v[k + j];
-    const int left = min(max(nv - k, 0), kAtOnce);
-    visit_km<kAtOnce, kCount>(g, lv, s, w, (1u << left) - 1u, edges);
-  }
-}
-
-template <typename T>
-__device__ T block_exclusive_scan(T x, T* total) {
-  __shared__ T wsum[32];
-  const uint32_t lane = lane_id();
-  const int w = threadIdx.x >> 5;
-  const int nw = blockDim.x >> 5;
-  T inc = x;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    T y = __shfl_up_sync(kFull, inc, o);
-    if ((int)lane >= o) inc += y;
-  }
-  if (lane == 31) wsum[w] = inc;
-  __syncthreads();
-  if (w == 0) {
-    T s = (int)lane < nw ? wsum[lane] : T(0);
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      T y = __shfl_up_sync(kFull, s, o);
-      if ((int)lane >= o) s += y;
-    }
-    if ((int)lane < nw) wsum[lane] = s;
-  }
-  __syncthreads();
-  const T base = w > 0 ? wsum[w - 1] : T(0);
-  *total = wsum[nw - 1];
-  __syncthreads();
-  return base + inc - x;
 }
 
 // ---------------------------------------------------------------------------
@@ -594,196 +453,6 @@ __device__ bool body_push_cta(const DevGraph& g, const Level& lv, const Stage& s
     }
   }
   return true;
-}
-
-// ---------------------------------------------------------------------------
-// Push, edge-centric (Section 3.1.1 edge list, restricted to the frontier's
-// edges): exclusive scan of the frontier degrees, then a load-balanced search
-// (merge path of the scan with the edge indices) gives every thread
-// kPeItems items (frontier boundaries or edges) regardless of degree skew.
-// ---------------------------------------------------------------------------
-__device__ void body_pe_reduce(const DevGraph& g, const Level& lv, const Buffers& b) {
-  const int f = lv.frontier;
-  const int nblk = (f + kPeTile - 1) / kPeTile;
-  for (int blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
-    long long sum = 0;
-    const int base = blk * kPeTile;
-#pragma unroll
-    for (int k = 0; k < kPeItems; ++k) {
-      const int i = base + k * kThreads + threadIdx.x;
-      if (i < f) {
-        const int32_t u = lv.qin[i];
-        const int32_t beg = g.off[u];
-        const int32_t d = g.off[u + 1] - beg;
-        b.pe_beg[i] = beg;
-        b.pe_scan[i] = d;
-        sum += d;
-      }
-    }
-    long long tot;
-    block_exclusive_scan<long long>(sum, &tot);
-    if (threadIdx.x == 0) b.pe_bsum[blk] = tot;
-  }
-}
-
-// One block.
-__device__ void body_pe_top(const Buffers& b, int f) {
-  const int nblk = (f + kPeTile - 1) / kPeTile;
-  long long carry = 0;
-  for (int base = 0; base < nblk; base += blockDim.x) {
-    const int i = base + threadIdx.x;
-    const long long x = i < nblk ? b.pe_bsum[i] : 0;
-    long long tot;
-    const long long ex = block_exclusive_scan<long long>(x, &tot);
-    if (i < nblk) b.pe_bsum[i] = carry + ex;
-    carry += tot;
-  }
-  if (threadIdx.x == 0) b.pe_bsum[nblk] = carry;
-}
-
-__device__ void body_pe_scan(const Buffers& b, int f) {
-  const int nblk = (f + kPeTile - 1) / kPeTile;
-  for (int blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
-    const int base = blk * kPeTile + threadIdx.x * kPeItems;
-    int32_t d[kPeItems];
-#pragma unroll
-    for (int k = 0; k < kPeItems; ++k) d[k] = (base + k < f) ? b.pe_scan[base + k] : 0;
-    int32_t run = 0;
-#pragma unroll
-    for (int k = 0; k < kPeItems; ++k) {
-      const int32_t t = d[k];
-      d[k] = run;
-      run += t;
-    }
-    long long tot;
-    const long long ex = block_exclusive_scan<long long>((long long)run, &tot);
-    const long long off = b.pe_bsum[blk] + ex;
-#pragma unroll
-    for (int k = 0; k < kPeItems; ++k)
-      if (base + k < f) b.pe_scan[base + k] = (int32_t)(off + d[k]);
-    if (blk == nblk - 1 && threadIdx.x == 0) b.pe_scan[f] = (int32_t)b.pe_bsum[nblk];
-  }
-}
-
-// A frontier of at most kPeSmall vertices fits one scan tile: every block then
-// scans the frontier degrees itself, in shared memory, and the level needs no
-// grid-wide scan phases (no extra grid barriers in the persistent kernel, no
-// work in the reduce/top/scan launches of the other drivers).
-constexpr int kPeSmall = kPeTile - 1;
-
-// s_a, s_beg: kPeTile + 1 entries. On return s_a[1 + i] is the exclusive scan
-// of the frontier degrees at i (s_a[1 + f] their total) and s_beg[1 + i] the
-// row start of frontier entry i; entry 0 of both is 0, the value the expand
-// uses before the first frontier entry. f <= kPeSmall.
-__device__ void pe_small_scan(const DevGraph& g, const Level& lv, int32_t* s_a, int32_t* s_beg) {
-  const int f = lv.frontier;
-  const int base = (int)threadIdx.x * kPeItems;
-  int32_t d[kPeItems];
-  int32_t run = 0;
-#pragma unroll
-  for (int k = 0; k < kPeItems; ++k) {
-    const int i = base + k;
-    int32_t deg = 0;
-    if (i < f) {
-      const int32_t u = lv.qin[i];
-      const int32_t b0 = g.off[u];
-      deg = g.off[u + 1] - b0;
-      s_beg[1 + i] = b0;
-    }
-    d[k] = run;
-    run += deg;
-  }
-  long long tot;
-  const long long ex = block_exclusive_scan<long long>((long long)run, &tot);
-#pragma unroll
-  for (int k = 0; k < kPeItems; ++k)
-    if (base + k < f) s_a[1 + base + k] = (int32_t)(ex + d[k]);
-  if (threadIdx.x == 0) {
-    s_a[0] = 0;
-    s_beg[0] = 0;
-    if (f <= kPeSmall) s_a[1 + f] = (int32_t)tot;  // callers guarantee it; the check keeps s_a in bounds
-  }
-  __syncthreads();
-}
-
-// Merge-path split: how many of the first d items of merge(A[0..na), j0+[0..nb))
-// are A items, with A first on ties (A[i] <= edge index => boundary first).
-__device__ __forceinline__ int merge_split(const int32_t* a, int na, long long j0, int nb, long long d) {
-  int lo = (int)max(0ll, d - nb), hi = (int)min(d, (long long)na);
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if ((long long)a[mid] <= j0 + d - 1 - mid)
-      lo = mid + 1;
-    else
-      hi = mid;
-  }
-  return lo;
-}
-
-// s_a, s_beg: kPeTile + 1 entries of shared memory each; s_split: 2 ints.
-// kSmall: the scan is already in s_a / s_beg (pe_small_scan), not in b.
-template <bool kSmall>
-__device__ void body_pe_expand(const DevGraph& g, const Level& lv, const Buffers& b, const Stage& stage,
-                               int32_t* s_a_buf, int32_t* s_beg_buf, int* s_split, unsigned long long& edges) {
-  const int f = lv.frontier;
-  const int32_t* scan = kSmall ? s_a_buf + 1 : b.pe_scan;
-  const int32_t E = scan[f];
-  const long long total = (long long)f + E;
-  // Tile length: a whole multiple of the block size, as short as spreads the
-  // items over every block (one per thread at least), at most kPeTile. A
-  // small level (a handful of frontier vertices with some thousands of edges)
-  // then runs on many blocks with an item or two per thread instead of a few
-  // full tiles, so its latency is one visit chain instead of eight.
-  const long long per_block = (total + gridDim.x - 1) / gridDim.x;
-  const int tile = (int)min((long long)kPeTile, max((long long)kThreads, (per_block + kThreads - 1) / kThreads * kThreads));
-  const int ipt = tile / kThreads;  // items per thread, 1..kPeItems
-  const long long ntiles = (total + tile - 1) / tile;
-  for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const long long d0 = t * tile;
-    const long long d1 = min(d0 + tile, total);
-    if (threadIdx.x < 2) s_split[threadIdx.x] = merge_split(scan, f, 0, E, threadIdx.x ? d1 : d0);
-    __syncthreads();
-    const int i0 = s_split[0], i1 = s_split[1];
-    const int na = i1 - i0;
-    const int tl = (int)(d1 - d0);
-    const int nb = tl - na;
-    const long long j0 = d0 - i0;
-    // s index k <-> frontier entry i0 - 1 + k (the vertex owning edge j0 may precede the tile)
-    const int32_t* s_a = s_a_buf;
-    const int32_t* s_beg = s_beg_buf;
-    if (kSmall) {
-      s_a = s_a_buf + i0;  // s_a_buf[1 + i] holds entry i, s_a_buf[0] the 0 before entry 0
-      s_beg = s_beg_buf + i0;
-    } else {
-      for (int k = threadIdx.x; k <= na; k += blockDim.x) {
-        const int gi = i0 - 1 + k;
-        s_a_buf[k] = gi >= 0 ? b.pe_scan[gi] : 0;
-        s_beg_buf[k] = gi >= 0 ? b.pe_beg[gi] : 0;
-      }
-      __syncthreads();
-    }
-    const int td0 = min((int)threadIdx.x * ipt, tl);
-    const int td1 = min(td0 + ipt, tl);
-    const int ti = merge_split(s_a + 1, na, j0, nb, td0);
-    int cur = ti;          // s index of the current vertex
-    int anext = ti + 1;    // s index of the next boundary
-    long long bj = j0 + (td0 - ti);
-    int32_t epos[kPeItems];
-    int ne = 0;
-    for (int step = td0; step < td1; ++step) {
-      if (anext <= na && (long long)s_a[anext] <= bj) {
-        cur = anext++;
-      } else {
-        epos[ne++] = s_beg[cur] + (int32_t)(bj - s_a[cur]);
-        ++bj;
-      }
-    }
-    int32_t v[kPeItems];
-#pragma unroll
-    for (int k = 0; k < kPeItems; ++k) v[k] = k < ne ? g.idx[epos[k]] : 0;
-    visit_k<kPeItems>(g, lv, stage, v, ne, edges);
-    stage_flush(stage, lv, 1);
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1163,6 +832,7 @@ __global__ void __launch_bounds__(kDecideThreads) k_decide(DevGraph g, Buffers b
     const unsigned long long e = *reinterpret_cast<volatile unsigned long long*>(&s.next_edges);
     s.next_count = 0;
     s.next_edges = 0;
+    s.heavy3[0] = 0;
     if (s.level >= 0 && s.variant == V_PULL) s.vsel ^= 1u;  // pull wrote the other bitmap
     s.qsel ^= 1u;
     L = s.level + 1;
@@ -1259,41 +929,31 @@ __global__ void __launch_bounds__(kThreads) k_push_cta(DevGraph g, Buffers b, Ru
   block_add_u64(edges, &st->next_edges);
 }
 
-// (A frontier of at most kPeSmall vertices is scanned by k_pe_expand itself:
-// the three scan launches then return at once.)
-__global__ void __launch_bounds__(kThreads) k_pe_reduce(DevGraph g, Buffers b, RunState* st) {
-  const Level lv = load_level(g, b, st);
-  if (lv.frontier <= kPeSmall) return;
-  body_pe_reduce(g, lv, b);
-}
-
-__global__ void __launch_bounds__(kThreads) k_pe_top(DevGraph g, Buffers b, RunState* st) {
-  (void)g;
-  const int f = st->frontier;
-  if (f <= kPeSmall) return;
-  body_pe_top(b, f);
-}
-
-__global__ void __launch_bounds__(kThreads) k_pe_scan(DevGraph g, Buffers b, RunState* st) {
-  (void)g;
-  const int f = st->frontier;
-  if (f <= kPeSmall) return;
-  body_pe_scan(b, f);
-}
-
-__global__ void __launch_bounds__(kThreads) k_pe_expand(DevGraph g, Buffers b, RunState* st) {
-  __shared__ int32_t s_a[kPeTile + 1];
-  __shared__ int32_t s_beg[kPeTile + 1];
-  __shared__ int s_split[2];
+__global__ void __launch_bounds__(kThreads) k_push_edge(DevGraph g, Buffers b, RunState* st) {
+  __shared__ int32_t s_a[kPeTile];
+  __shared__ int32_t s_beg[kPeTile];
   BFS_DECLARE_STAGE(stage);
   const Level lv = load_level(g, b, st);
   unsigned long long edges = 0;
-  if (lv.frontier <= kPeSmall) {
-    pe_small_scan(g, lv, s_a, s_beg);
-    body_pe_expand<true>(g, lv, b, stage, s_a, s_beg, s_split, edges);
-  } else {
-    body_pe_expand<false>(g, lv, b, stage, s_a, s_beg, s_split, edges);
-  }
+  if (lv.shared_scan)
+    body_push_shared(g, lv, lv.qin, lv.frontier, stage, s_a, s_beg, edges);
+  else
+    body_push_tiles(g, lv, stage, s_a, s_beg, b.heavy, b.heavy_cap, edges);
+  stage_flush(stage, lv, 1);
+  block_add_u64(edges, &st->next_edges);
+}
+
+// (Returns at once when nothing was set aside.)
+__global__ void __launch_bounds__(kThreads) k_push_heavy(DevGraph g, Buffers b, RunState* st) {
+  __shared__ int32_t s_a[kPeTile];
+  __shared__ int32_t s_beg[kPeTile];
+  const unsigned int count = st->heavy3[0];
+  if (count == 0u) return;
+  BFS_DECLARE_STAGE(stage);
+  const Level lv = load_level(g, b, st);
+  unsigned long long edges = 0;
+  body_push_heavy(g, lv, stage, s_a, s_beg, b.heavy, (int32_t)min(count, (unsigned)b.heavy_cap), edges);
+  stage_flush(stage, lv, 1);
   block_add_u64(edges, &st->next_edges);
 }
 
@@ -1375,8 +1035,10 @@ __device__ __forceinline__ Level persistent_level(const DevGraph& g, const Buffe
   lv.vis_next = vsel ? b.vis[0] : b.vis[1];
   lv.depth = depth;
   lv.tail = &st->tail3[slot];
+  lv.n_heavy = &st->heavy3[slot];
   lv.next_depth = L + 1;
   lv.frontier = (int32_t)f;
+  lv.shared_scan = pe_shared(f, (long long)e, g.gfeat[F_DEG_MAX] >= kHeavy);
   lv.latency_bound = (long long)e < kLatencyEdges;
   lv.pull_sparse = (long long)g.n_active - discovered < (long long)(g.n_active >> 4);
   return lv;
@@ -1388,26 +1050,22 @@ __device__ __forceinline__ Level persistent_level(const DevGraph& g, const Buffe
 __device__ __forceinline__ unsigned long long persistent_level_work(const DevGraph& g, const Buffers& b, RunState* st,
                                                                     const Level& lv, int32_t v, int32_t vw,
                                                                     const Stage& stage, CtaPipe& pp, int32_t* ubuf,
-                                                                    int* s_split, unsigned long long& bar_target) {
-  const unsigned int f = (unsigned int)lv.frontier;
+                                                                    unsigned long long& bar_target) {
   unsigned long long edges = 0;
   switch (v) {
     case V_PUSH_THREAD: body_push_thread(g, lv, stage, edges); break;
     case V_PUSH_WARP: body_push_warp(g, lv, stage, vw, edges); break;
     case V_PUSH_CTA: body_push_cta(g, lv, stage, pp, &st->status, edges); break;
     case V_PUSH_EDGE:
-      if ((int)f <= kPeSmall) {
-        pe_small_scan(g, lv, ubuf, ubuf + kPeSlot);
-        body_pe_expand<true>(g, lv, b, stage, ubuf, ubuf + kPeSlot, s_split, edges);
+      if (lv.shared_scan) {
+        body_push_shared(g, lv, lv.qin, lv.frontier, stage, ubuf, ubuf + kPeSlot, edges);
         break;
       }
-      body_pe_reduce(g, lv, b);
+      body_push_tiles(g, lv, stage, ubuf, ubuf + kPeSlot, b.heavy, b.heavy_cap, edges);
+      if (g.gfeat[F_DEG_MAX] < kHeavy) break;  // nothing can have been set aside
       if (!grid_arrive_wait(&st->bar64, bar_target, &st->status)) break;
-      if (blockIdx.x == 0) body_pe_top(b, (int)f);
-      if (!grid_arrive_wait(&st->bar64, bar_target, &st->status)) break;
-      body_pe_scan(b, (int)f);
-      if (!grid_arrive_wait(&st->bar64, bar_target, &st->status)) break;
-      body_pe_expand<false>(g, lv, b, stage, ubuf, ubuf + kPeSlot, s_split, edges);
+      body_push_heavy(g, lv, stage, ubuf, ubuf + kPeSlot, b.heavy,
+                      (int32_t)min(*reinterpret_cast<volatile unsigned int*>(lv.n_heavy), (unsigned)b.heavy_cap), edges);
       break;
     case V_EDGE_LIST: body_edge_list<false>(g, lv, stage, edges); break;
     case V_REV_EDGE_LIST: body_edge_list<true>(g, lv, stage, edges); break;
@@ -1492,6 +1150,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_bfs_persistent(const __grid_con
     for (int k = 0; k < 3; ++k) {
       st->tail3[k] = 0;
       st->edg3[k] = 0;
+      st->heavy3[k] = 0;
     }
     st->small_tail = 0;
     st->small_seq = 0;
@@ -1501,7 +1160,6 @@ __global__ void __launch_bounds__(kThreads, 4) k_bfs_persistent(const __grid_con
   __shared__ alignas(128) int32_t ubuf[2 * kPeSlot];
   static_assert(2 * kPeSlot >= 4 * kCandCap && kStageCap >= kWonCap, "the leader's queues");
   __shared__ alignas(8) uint64_t bar[2];
-  __shared__ int s_split[2];
   __shared__ SmallShared s_small;
   __shared__ RunLog s_log;
   // the tree is evaluated by every warp every level: its bit-parallel form
@@ -1598,12 +1256,13 @@ __global__ void __launch_bounds__(kThreads, 4) k_bfs_persistent(const __grid_con
         const uint32_t after = next == 2u ? 0u : next + 1u;
         st->tail3[after] = 0;  // the slot of a barrier every block has left
         st->edg3[after] = 0;
+        st->heavy3[after] = 0;
       }
       if (threadIdx.x == kThreads - 1) log_level(s_log, L, v, f, (long long)e);
     }
     const Level lv = persistent_level(g, b, st, depth, L, f, e, discovered, vsel, next);
     const int32_t vw = warp_width(f, (long long)e, g.vw_policy);
-    const unsigned long long e_block = persistent_level_work(g, b, st, lv, v, vw, stage, pp, ubuf, s_split, bar_target);
+    const unsigned long long e_block = persistent_level_work(g, b, st, lv, v, vw, stage, pp, ubuf, bar_target);
     if (v == V_PULL) vsel ^= 1u;
     prev = v;
     ok = level_arrive_wait(&st->tail3[next], &st->edg3[next], e_block, &st->status, &f, &e,
@@ -1652,7 +1311,7 @@ __global__ void __launch_bounds__(kThreads) k_small_levels(const __grid_constant
     mbar_fence_init();
   }
   cluster_barrier();  // the state is read and every block's mbarriers are ready
-  const Buffers swapped{{b.q[1], b.q[0]}, {b.vis[0], b.vis[1]}, b.pe_scan, b.pe_beg, b.pe_bsum, b.pe_blocks_cap, 0};
+  const Buffers swapped{{b.q[1], b.q[0]}, {b.vis[0], b.vis[1]}, b.heavy, b.heavy_cap, 0};
   small_run<kRecord>(g, swapped, vsel ? b.vis[1] : b.vis[0], st->depth, st, tc.qs, tc.tree, tc.nodes, s_log,
                      s_small, ubuf, sbuf, v);
   if (cluster_rank() == 0u && threadIdx.x == 0 && s_small.out.L > L) {
@@ -1691,7 +1350,6 @@ __global__ void __launch_bounds__(kThreads, 4) k_profile_level(DevGraph g, Buffe
                                                             long long discovered, uint32_t vsel) {
   __shared__ alignas(128) int32_t ubuf[2 * kPeSlot];
   __shared__ alignas(8) uint64_t bar[2];
-  __shared__ int s_split[2];
   BFS_DECLARE_STAGE(stage);
   cta_pipe_init(bar);
   CtaPipe pp{ubuf, bar, 0u, 0u, 0u};
@@ -1700,7 +1358,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_profile_level(DevGraph g, Buffe
   if (!grid_arrive_wait(&st->bar64, bar_target, &st->status)) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) st->prof_t0 = (long long)global_ns();
   const Level lv = persistent_level(g, b, st, depth, L, f, e, discovered, vsel, (uint32_t)((L + 1) % 3));
-  const unsigned long long e_block = persistent_level_work(g, b, st, lv, v, vw, stage, pp, ubuf, s_split, bar_target);
+  const unsigned long long e_block = persistent_level_work(g, b, st, lv, v, vw, stage, pp, ubuf, bar_target);
   unsigned int fn = 0;
   unsigned long long en = 0;
   if (!level_arrive_wait(&st->tail3[(L + 1) % 3], &st->edg3[(L + 1) % 3], e_block, &st->status, &fn, &en)) return;
@@ -1718,6 +1376,7 @@ __global__ void k_profile_reset(RunState* st, int32_t slot) {
   st->status = ST_OK;
   st->tail3[slot] = 0;
   st->edg3[slot] = 0;
+  st->heavy3[slot] = 0;
 }
 
 // Undo a profiled level in the persistent layout: the `count` vertices it

@@ -10,8 +10,10 @@ constexpr int kMaxCluster = 16;   // blocks of a cluster that runs small levels 
 constexpr int kDecideThreads = 32;  // block size of k_decide: one warp evaluates the bit-parallel tree
 constexpr int kCtaChunk = 2048;   // int32 per shared-memory stage of the CTA variant (8 KB)
 constexpr int kCtaDirect = 512;   // adjacency shorter than this is read directly, not staged
-constexpr int kPeItems = 8;       // items per thread in the edge-centric scan / expand
-constexpr int kPeTile = kThreads * kPeItems;  // frontier entries per scan block, items per expand tile
+constexpr int kPeItems = 8;       // entries per thread in a scan
+constexpr int kPeTile = kThreads * kPeItems;  // entries per block of a scan
+constexpr int kHeavy = 1024;        // degree from which an edge-centric level deals a vertex over all blocks
+constexpr int kHeavyCap = 1 << 16;  // most vertices an edge-centric level sets aside
 
 __global__ void k_init(DevGraph g, Buffers b, RunState* st, int32_t* depth, int32_t root, int32_t forced,
                        const TreeNode* tree, int32_t tree_nodes, const QsTree* tree_qs, int32_t use_handles);
@@ -20,10 +22,8 @@ __global__ void k_loop_start(DevGraph g, Buffers b, RunState* st);
 __global__ void k_push_thread(DevGraph g, Buffers b, RunState* st);
 __global__ void k_push_warp(DevGraph g, Buffers b, RunState* st);
 __global__ void k_push_cta(DevGraph g, Buffers b, RunState* st);
-__global__ void k_pe_reduce(DevGraph g, Buffers b, RunState* st);
-__global__ void k_pe_top(DevGraph g, Buffers b, RunState* st);
-__global__ void k_pe_scan(DevGraph g, Buffers b, RunState* st);
-__global__ void k_pe_expand(DevGraph g, Buffers b, RunState* st);
+__global__ void k_push_edge(DevGraph g, Buffers b, RunState* st);
+__global__ void k_push_heavy(DevGraph g, Buffers b, RunState* st);
 __global__ void k_pull(DevGraph g, Buffers b, RunState* st);
 // Vertex push appending by CM_WARP or CM_ATOMIC (count-mode comparison)
 __global__ void k_push_thread_warp_count(DevGraph g, Buffers b, RunState* st);
