@@ -336,8 +336,8 @@ int bfs_batch_tune_ex(bfs_graph_t g, const int32_t* roots, int32_t k, int32_t* d
  * owns, and gets the same depths as bfs_run.
  *
  * Limit: n <= 1,048,576 vertices; larger n returns BFS_ERR_INVALID_ARG. The
- * traversal's scratch (two frontier queues, the visited bitmap, counters) is a
- * fixed device array of about 8.1 MB inside the library, held by every GPU that
+ * traversal's scratch (two frontier queues, the visited bitmap, a list, counters) is a
+ * fixed device array of about 8.2 MB inside the library, held by every GPU that
  * loads the library until the process exits. Every call looks up that array's
  * device address in the current device's context (cudaGetSymbolAddress, which
  * allocates nothing), so a device reset between calls leaves no stale address;
@@ -349,9 +349,10 @@ int bfs_batch_tune_ex(bfs_graph_t g, const int32_t* roots, int32_t k, int32_t* d
  * the one array, which keeps the previous call's contents (each call clears
  * what it reads first): calls whose work overlaps on the GPU, from any stream
  * or thread, race and corrupt each other, so serialise them. The CSR is
- * validated on every call (BFS_ERR_BAD_GRAPH). Synchronous: the level loop
- * reads each level's frontier size back to the host. Uses a simple one thread
- * per frontier vertex push for every level (no tree switching).
+ * validated on every call (BFS_ERR_BAD_GRAPH). Synchronous: one cooperative
+ * launch validates and traverses, then its status is read back. Every level is
+ * the edge-centric push (no tree switching). BFS_ERR_TIMEOUT if a bounded
+ * device-side wait gave up.
  */
 int bfs_run_static(const int32_t* row_offsets, const int32_t* col_indices, int64_t n, int64_t m, int32_t root,
                    int32_t* depth_out, bfs_stream_t stream);

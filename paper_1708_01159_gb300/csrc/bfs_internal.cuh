@@ -566,13 +566,4 @@ __device__ __forceinline__ bool level_arrive_wait(unsigned long long* tail, unsi
   return ok;
 }
 
-// Try to claim vertex v: set its visited bit. True only for the one thread
-// whose atomicOr flipped the bit, so each vertex enters the queue once.
-__device__ __forceinline__ bool claim(uint32_t* vis, int32_t v) {
-  const uint32_t bit = 1u << (v & 31);
-  uint32_t* w = vis + (v >> 5);
-  if (*reinterpret_cast<volatile uint32_t*>(w) & bit) return false;  // cheap filter; bits only go 0 -> 1
-  return (atomicOr(w, bit) & bit) == 0u;
-}
-
 }  // namespace bfs

@@ -1,6 +1,7 @@
 """The edge-centric push at the edges of its tiles and lists: degrees around the
 heavy threshold (1024), frontiers around one scan tile (2048) and one block's
-tile (32 to 256). Depths equal the oracle's."""
+tile (32 to 256), a heavy list that overflows (the allocation-free entry point's
+16,384 vertices) and a CSR at an unaligned address. Depths equal the oracle's."""
 import numpy as np
 import pytest
 
@@ -58,3 +59,17 @@ def test_edge_centric_push_matches_the_oracle(name):
             assert np.array_equal(d.cpu().numpy(), ref.depth), (mode, blocks)
             assert st["edges_reached"] == ref.edges_reached
             assert np.array_equal(st["frontier"], ref.level_count)
+
+
+@pytest.mark.parametrize("name", sorted(CASES) + ["list overflows"])
+def test_allocation_free_entry_matches_the_oracle(name):
+    g = fan(17000, [1024], 40000) if name == "list overflows" else CASES[name]()
+    ref = oracle.bfs(g.off, g.idx, 0)
+    for shift in (0, 1, 3):  # entries the arrays are off a 16-byte boundary
+        off = torch.zeros(g.n + 1 + shift, dtype=torch.int32, device="cuda")[shift:]
+        idx = torch.zeros(max(g.m, 1) + shift, dtype=torch.int32, device="cuda")[shift:]
+        out = torch.full((g.n + shift,), 7, dtype=torch.int32, device="cuda")[shift:]
+        off.copy_(torch.from_numpy(g.off))
+        idx[:g.m].copy_(torch.from_numpy(g.idx))
+        bfs.bfs_run_static(off, idx[:g.m], 0, out)
+        assert np.array_equal(out.cpu().numpy(), ref.depth), shift
