@@ -689,8 +689,8 @@ int ensure_origin(bfs_graph* g) {
   cudaStream_t s;
   CU(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
   const int blocks = g->sms * 4;
-  k_build_origin<<<blocks, kThreads, 0, s>>>(g->dg.off, g->dg.n, out);
-  if (!g->symmetric) k_build_origin<<<blocks, kThreads, 0, s>>>(g->dg.in_off, g->dg.n, in);
+  k_build_origin<<<blocks, kThreads, 0, s>>>(g->dg.off, g->dg.n, g->dg.m, out);
+  if (!g->symmetric) k_build_origin<<<blocks, kThreads, 0, s>>>(g->dg.in_off, g->dg.n, g->dg.m, in);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   cudaStreamDestroy(s);
@@ -1018,37 +1018,45 @@ int bfs::batch_async(bfs_graph* g, MsSet* set, const int32_t* roots, int32_t k, 
 
 namespace {
 
-// The 5-number summary (nearest rank) and floor(256 sd) of the degrees of all
-// n vertices, on the device: the row lengths of `off`, plus those of `off2`
-// when given (in + out = total degree). Synchronous.
-int degree_summary(const int32_t* off, const int32_t* off2, int32_t n, int blocks, long long out6[6]) {
-  unsigned int* mm = nullptr;  // [0] min, [1] max
-  unsigned long long* sums = nullptr;
+// The 5-number summaries (nearest rank) and floor(256 sd) of the out-, in- and
+// total degrees of all n vertices, on the device: the row lengths of `off`, of
+// `off_in` (null: a symmetric graph) and their sums. Synchronous.
+int degree_summaries(const int32_t* off, const int32_t* off_in, int32_t n, int blocks, long long out6[6],
+                     long long in6[6], long long tot6[6]) {
+  struct Block {
+    DegSums sums[3];
+    long long out[18];
+  };
+  Block* d = nullptr;
+  Block h{};
   int32_t* hist = nullptr;
-  long long* st6 = nullptr;
-  unsigned int mm_h[2] = {0xffffffffu, 0u};
-  cudaError_t e = cudaMalloc(&mm, 8);
-  if (e == cudaSuccess) e = cudaMalloc(&sums, 16);
-  if (e == cudaSuccess) e = cudaMalloc(&st6, 6 * 8);
-  if (e == cudaSuccess) e = cudaMemcpy(mm, mm_h, 8, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemset(sums, 0, 16);
+  cudaError_t e = cudaMalloc(&d, sizeof(Block));
+  if (e == cudaSuccess) e = cudaMemset(d, 0, sizeof(Block));
   if (e == cudaSuccess) {
-    k_deg_reduce<<<blocks, kThreads>>>(off, off2, n, sums, sums + 1, mm, mm + 1);
-    e = cudaMemcpy(mm_h, mm, 8, cudaMemcpyDeviceToHost);
+    k_deg_reduce<<<blocks, kThreads>>>(off, off_in, n, d->sums);
+    e = cudaMemcpy(&h, d, sizeof h.sums, cudaMemcpyDeviceToHost);
   }
-  if (e == cudaSuccess) e = cudaMalloc(&hist, ((size_t)mm_h[1] + 1) * 4);
-  if (e == cudaSuccess) e = cudaMemset(hist, 0, ((size_t)mm_h[1] + 1) * 4);
+  // the kinds' histograms one after another
+  const long long at1 = (long long)h.sums[0].dmax + 1, at2 = at1 + (long long)h.sums[1].dmax + 1;
+  const size_t bins = (size_t)(off_in ? at2 + (long long)h.sums[2].dmax + 1 : at1);
+  if (e == cudaSuccess) e = cudaMalloc(&hist, bins * 4);
+  if (e == cudaSuccess) e = cudaMemset(hist, 0, bins * 4);
   if (e == cudaSuccess) {
-    k_deg_hist<<<blocks, kThreads>>>(off, off2, n, hist);
-    k_deg_finish<<<1, kThreads>>>(hist, (int64_t)mm_h[1], n, sums, sums + 1, st6);
-    e = cudaMemcpy(out6, st6, 6 * 8, cudaMemcpyDeviceToHost);
+    k_deg_hist<<<blocks, kThreads>>>(off, off_in, n, at1, at2, hist);
+    k_deg_finish<<<off_in ? 3 : 2, kDegFinishThreads>>>(hist, at1, at2, n, d->sums, off_in ? 0 : 1, d->out);
+    e = cudaMemcpy(h.out, d->out, sizeof h.out, cudaMemcpyDeviceToHost);
   }
-  for (void* p : {(void*)mm, (void*)sums, (void*)hist, (void*)st6})
-    if (p) cudaFree(p);
+  if (d) cudaFree(d);
+  if (hist) cudaFree(hist);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return fail(e == cudaErrorMemoryAllocation ? BFS_ERR_OOM : BFS_ERR_CUDA, "degree statistics: %s",
                 cudaGetErrorString(e));
+  }
+  for (int k = 0; k < 6; ++k) {
+    out6[k] = h.out[k];
+    in6[k] = off_in ? h.out[6 + k] : h.out[k];
+    tot6[k] = off_in ? h.out[12 + k] : h.out[6 + k];
   }
   return BFS_OK;
 }
@@ -1296,7 +1304,7 @@ int bfs_graph_create(const int32_t* row_offsets, const int32_t* col_indices, int
         e = cudaMemcpy(cnt, in_off, (n + 1) * 4, cudaMemcpyDeviceToDevice);
       }
       if (e == cudaSuccess) {
-        k_tr_scatter<<<blocks, kThreads>>>(off, idx, (int32_t)n, cnt, in_idx);
+        k_tr_scatter<<<g->sms * 8, kThreads>>>(off, idx, (int32_t)n, (int32_t)m, cnt, in_idx);
         e = cudaDeviceSynchronize();
       }
       if (e != cudaSuccess) r = fail(BFS_ERR_CUDA, "transpose: %s", cudaGetErrorString(e));
@@ -1346,9 +1354,8 @@ int bfs_graph_create(const int32_t* row_offsets, const int32_t* col_indices, int
   }
   // degree statistics (Section 4.1 degree distribution): out-degree, in-degree
   // (the transpose's row lengths) and total degree
-  r = degree_summary(off, nullptr, (int32_t)n, blocks, g->stats6);
-  if (r == BFS_OK) r = degree_summary(in_off, nullptr, (int32_t)n, blocks, g->stats_in6);
-  if (r == BFS_OK) r = degree_summary(off, in_off, (int32_t)n, blocks, g->stats_tot6);
+  r = degree_summaries(off, g->symmetric ? nullptr : in_off, (int32_t)n, blocks, g->stats6, g->stats_in6,
+                       g->stats_tot6);
   if (r != BFS_OK) {
     cleanup();
     return r;

@@ -975,11 +975,56 @@ __global__ void __launch_bounds__(kThreads) k_rev_edge_list(DevGraph g, Buffers 
   block_add_u64(edges, &st->next_edges);
 }
 
-// Origin of every CSR entry: the vertex whose row [off[v], off[v + 1]) holds it.
-__global__ void k_build_origin(const int32_t* off, int32_t n, int32_t* origin) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride)
-    for (int32_t e = off[v]; e < off[v + 1]; ++e) origin[e] = (int32_t)v;
+// fn(e, v) for every CSR entry e and the vertex v whose row [off[v], off[v + 1])
+// holds it. A block takes kPeTile consecutive entries, finds the rows that hold
+// them and each entry's row by binary search (in shared memory unless empty
+// rows make them many), so a hub's row is shared out like any other. (A thread
+// per row spent 19.9 ms in the transpose of a directed R-MAT graph of 2^20
+// vertices and 15.9M edges, walking its longest row; creation with one traversal
+// takes 2.2 ms in all with this and the summaries in one pass, 24.1 before.)
+template <typename Fn>
+__device__ __forceinline__ void for_each_entry(const int32_t* off, int32_t n, int32_t m, Fn fn) {
+  __shared__ int32_t s_off[kPeTile];
+  __shared__ int32_t s_row[2];
+  for (long long c0 = (long long)blockIdx.x * kPeTile; c0 < m; c0 += (long long)gridDim.x * kPeTile) {
+    const int32_t c1 = (int32_t)min(c0 + kPeTile, (long long)m);
+    if (threadIdx.x < 2) {  // the last row that starts at or before the chunk's first / last entry
+      const int32_t e = threadIdx.x ? c1 - 1 : (int32_t)c0;
+      int32_t lo = 0, hi = n - 1;
+      while (lo < hi) {
+        const int32_t mid = lo + (hi - lo + 1) / 2;
+        if (off[mid] <= e)
+          lo = mid;
+        else
+          hi = mid - 1;
+      }
+      s_row[threadIdx.x] = lo;
+    }
+    __syncthreads();
+    const int32_t r0 = s_row[0], rows = s_row[1] - r0 + 1;
+    const bool shared = rows <= kPeTile;  // uniform
+    if (shared)
+      for (int32_t r = threadIdx.x; r < rows; r += blockDim.x) s_off[r] = off[r0 + r];
+    __syncthreads();
+    const int32_t* start = shared ? s_off : off + r0;
+    for (int32_t e = (int32_t)c0 + (int32_t)threadIdx.x; e < c1; e += blockDim.x) {
+      int32_t lo = 0, hi = rows - 1;
+      while (lo < hi) {
+        const int32_t mid = lo + (hi - lo + 1) / 2;
+        if (start[mid] <= e)
+          lo = mid;
+        else
+          hi = mid - 1;
+      }
+      fn(e, r0 + lo);
+    }
+    __syncthreads();
+  }
+}
+
+// Origin of every CSR entry: the vertex whose row holds it.
+__global__ void __launch_bounds__(kThreads) k_build_origin(const int32_t* off, int32_t n, int32_t m, int32_t* origin) {
+  for_each_entry(off, n, m, [=](int32_t e, int32_t v) { origin[e] = v; });
 }
 
 __global__ void __launch_bounds__(kThreads) k_pull(DevGraph g, Buffers b, RunState* st) {
@@ -1408,44 +1453,72 @@ __global__ void k_validate(const int32_t* off, const int32_t* idx, int32_t n, in
   if (my) atomicOr(bad, 1);
 }
 
-// Degree of v for the statistics: the row length in `off`, plus the row
-// length in `off2` when given (in-degree + out-degree = total degree).
-__device__ __forceinline__ unsigned int stat_degree(const int32_t* off, const int32_t* off2, int64_t v) {
-  unsigned int d = (unsigned int)(off[v + 1] - off[v]);
-  if (off2) d += (unsigned int)(off2[v + 1] - off2[v]);
-  return d;
+// Degrees for the statistics: out (row length in off), in (in off_in) and
+// total, three summaries in one pass over the vertices; off_in null for a
+// symmetric graph, whose in-degree summary is its out-degree one and whose
+// total degrees are twice the out-degrees, so that only the first is taken.
+__device__ __forceinline__ void stat_degrees(const int32_t* off, const int32_t* off_in, int64_t v, unsigned int (&d)[3]) {
+  d[0] = (unsigned int)(off[v + 1] - off[v]);
+  d[1] = off_in ? (unsigned int)(off_in[v + 1] - off_in[v]) : 0u;
+  d[2] = d[0] + d[1];
 }
 
-__global__ void k_deg_reduce(const int32_t* off, const int32_t* off2, int32_t n, unsigned long long* s1,
-                             unsigned long long* s2, unsigned int* dmin, unsigned int* dmax) {
+// Sums, sums of squares, minima and maxima of the (up to) three degrees.
+__global__ void __launch_bounds__(kThreads) k_deg_reduce(const int32_t* off, const int32_t* off_in, int32_t n,
+                                                         DegSums* out) {
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  unsigned long long a = 0, q = 0;
-  unsigned int lo = 0xffffffffu, hi = 0;
+  const int kinds = off_in ? 3 : 1;
+  unsigned long long a[3] = {0, 0, 0}, q[3] = {0, 0, 0};
+  unsigned int hi[3] = {0, 0, 0};
   for (int64_t v = tid; v < n; v += stride) {
-    const unsigned int d = stat_degree(off, off2, v);
-    a += (unsigned long long)d;
-    q += (unsigned long long)d * (unsigned long long)d;
-    lo = min(lo, d);
-    hi = max(hi, d);
-  }
-  block_add_u64(a, s1);
-  block_add_u64(q, s2);
+    unsigned int d[3];
+    stat_degrees(off, off_in, v, d);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    lo = min(lo, __shfl_xor_sync(kFull, lo, o));
-    hi = max(hi, __shfl_xor_sync(kFull, hi, o));
+    for (int k = 0; k < 3; ++k) {
+      a[k] += (unsigned long long)d[k];
+      q[k] += (unsigned long long)d[k] * (unsigned long long)d[k];
+      hi[k] = max(hi[k], d[k]);
+    }
   }
-  if (lane_id() == 0) {
-    atomicMin(dmin, lo);
-    atomicMax(dmax, hi);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    if (k >= kinds) break;  // uniform
+    block_add_u64(a[k], &out[k].s1);
+    block_add_u64(q[k], &out[k].s2);
+    const unsigned int h = __reduce_max_sync(kFull, hi[k]);
+    if (lane_id() == 0) atomicMax(&out[k].dmax, h);
   }
 }
 
-__global__ void k_deg_hist(const int32_t* off, const int32_t* off2, int32_t n, int32_t* hist) {
-  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// Histograms of the degrees, kind k's at hist + at[k]. Degrees below kDegShared
+// are counted in shared memory first (most vertices share a few small degrees).
+constexpr int kDegShared = 512;
+__global__ void __launch_bounds__(kThreads) k_deg_hist(const int32_t* off, const int32_t* off_in, int32_t n,
+                                                       long long at1, long long at2, int32_t* hist) {
+  __shared__ int32_t s_hist[3 * kDegShared];
+  const int kinds = off_in ? 3 : 1;
+  for (int i = threadIdx.x; i < 3 * kDegShared; i += blockDim.x) s_hist[i] = 0;
+  __syncthreads();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t v = tid; v < n; v += stride) atomicAdd(&hist[stat_degree(off, off2, v)], 1);
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
+    unsigned int d[3];
+    stat_degrees(off, off_in, v, d);
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      if (k < kinds) {
+        if (d[k] < (unsigned)kDegShared)
+          atomicAdd(&s_hist[k * kDegShared + d[k]], 1);
+        else
+          atomicAdd(&hist[(k == 0 ? 0 : k == 1 ? at1 : at2) + d[k]], 1);
+      }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < kinds * kDegShared; i += blockDim.x)
+    if (s_hist[i]) {
+      const int kk = i / kDegShared;
+      atomicAdd(&hist[(kk == 0 ? 0 : kk == 1 ? at1 : at2) + i % kDegShared], s_hist[i]);
+    }
 }
 
 namespace {
@@ -1463,34 +1536,50 @@ __device__ unsigned long long isqrt_u128(unsigned __int128 x) {
 }
 }  // namespace
 
-// One block: 5-number summary by nearest rank (q_k = sorted[floor(k (n-1)/4)])
-// from the degree histogram, and floor(256 sigma) exactly:
-// isqrt(65536 (n S2 - S1^2)) / n.
-__global__ void k_deg_finish(const int32_t* hist, int64_t maxdeg, int32_t n, const unsigned long long* s1p,
-                             const unsigned long long* s2p, long long* out6) {
+// Block b: 5-number summary by nearest rank (q_k = sorted[floor(k (n-1)/4)])
+// from kind b's degree histogram, and floor(256 sigma) exactly: isqrt(65536 (n
+// S2 - S1^2)) / n. symmetric: block 1 gives the total degree's summary, whose
+// values are twice the out-degree's.
+constexpr int kDegItems = 4;
+__global__ void __launch_bounds__(kDegFinishThreads) k_deg_finish(const int32_t* hist, long long at1, long long at2,
+                                                                  int32_t n, const DegSums* sums, int32_t symmetric,
+                                                                  long long* out) {
   __shared__ long long carry_s;
+  const int kind = symmetric ? 0 : (int)blockIdx.x;
+  const long long twice = symmetric && blockIdx.x == 1 ? 2 : 1;
+  const int32_t* h = hist + (kind == 0 ? 0 : kind == 1 ? at1 : at2);
+  const long long maxdeg = sums[kind].dmax;
+  long long* out6 = out + 6 * blockIdx.x;
   long long rank[5];
 #pragma unroll
   for (int k = 0; k < 5; ++k) rank[k] = ((long long)k * (n - 1)) / 4;
   if (threadIdx.x == 0) carry_s = 0;
   __syncthreads();
-  for (int64_t base = 0; base <= maxdeg; base += blockDim.x) {
-    const int64_t d = base + threadIdx.x;
-    const long long c = d <= maxdeg ? hist[d] : 0;
-    long long tot;
-    const long long ex = block_exclusive_scan<long long>(c, &tot);
-    const long long before = carry_s + ex;  // vertices with degree < d
-    // d is the k-th quantile when before <= rank_k < before + c
+  for (long long base = 0; base <= maxdeg; base += (long long)blockDim.x * kDegItems) {
+    const long long d0 = base + (long long)threadIdx.x * kDegItems;
+    long long c[kDegItems], sum = 0;
 #pragma unroll
-    for (int k = 0; k < 5; ++k)
-      if (c > 0 && before <= rank[k] && rank[k] < before + c) out6[k] = d;
+    for (int i = 0; i < kDegItems; ++i) {
+      c[i] = d0 + i <= maxdeg ? h[d0 + i] : 0;
+      sum += c[i];
+    }
+    long long tot;
+    long long before = carry_s + block_exclusive_scan<long long>(sum, &tot);  // vertices with degree < d0
+#pragma unroll
+    for (int i = 0; i < kDegItems; ++i) {
+      // d is the k-th quantile when before <= rank_k < before + c
+#pragma unroll
+      for (int k = 0; k < 5; ++k)
+        if (c[i] > 0 && before <= rank[k] && rank[k] < before + c[i]) out6[k] = twice * (d0 + i);
+      before += c[i];
+    }
     __syncthreads();
     if (threadIdx.x == 0) carry_s += tot;
     __syncthreads();
   }
   if (threadIdx.x == 0) {
-    const unsigned __int128 S1 = *s1p, S2 = *s2p;
-    const unsigned __int128 var_n2 = (unsigned __int128)n * S2 - S1 * S1;
+    const unsigned __int128 S1 = sums[kind].s1, S2 = sums[kind].s2;
+    const unsigned __int128 var_n2 = ((unsigned __int128)n * S2 - S1 * S1) * (unsigned)(twice * twice);
     out6[5] = (long long)(isqrt_u128(var_n2 * 65536u) / (unsigned long long)n);
   }
 }
@@ -1556,14 +1645,9 @@ __global__ void __launch_bounds__(kThreads) k_scan_apply(const int32_t* in, int3
   }
 }
 
-__global__ void k_tr_scatter(const int32_t* off, const int32_t* idx, int32_t n, int32_t* cursor, int32_t* in_idx) {
-  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t u = tid; u < n; u += stride)
-    for (int32_t e = off[u]; e < off[u + 1]; ++e) {
-      const int32_t v = idx[e];
-      in_idx[atomicAdd(&cursor[v], 1)] = (int32_t)u;
-    }
+__global__ void __launch_bounds__(kThreads) k_tr_scatter(const int32_t* off, const int32_t* idx, int32_t n, int32_t m,
+                                                          int32_t* cursor, int32_t* in_idx) {
+  for_each_entry(off, n, m, [=](int32_t e, int32_t v) { in_idx[atomicAdd(&cursor[idx[e]], 1)] = v; });
 }
 
 // Bit v of the starting bitmap: set iff v has neither in- nor out-edges. No

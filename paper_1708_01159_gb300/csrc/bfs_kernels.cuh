@@ -30,7 +30,7 @@ __global__ void k_push_thread_warp_count(DevGraph g, Buffers b, RunState* st);
 __global__ void k_push_thread_atomic_count(DevGraph g, Buffers b, RunState* st);
 __global__ void k_edge_list(DevGraph g, Buffers b, RunState* st);
 __global__ void k_rev_edge_list(DevGraph g, Buffers b, RunState* st);
-__global__ void k_build_origin(const int32_t* off, int32_t n, int32_t* origin);
+__global__ void k_build_origin(const int32_t* off, int32_t n, int32_t m, int32_t* origin);
 __global__ void k_undo_level(Buffers b, RunState* st);
 // The persistent traversal kernel for graphs with vertex records of the given
 // width (0: none); parameters DevGraph, Buffers, RunState*, depth, root, forced,
@@ -46,17 +46,23 @@ __global__ void k_undo_level_p(Buffers b, int32_t* depth, uint32_t qout, unsigne
 
 // graph creation
 __global__ void k_validate(const int32_t* off, const int32_t* idx, int32_t n, int32_t m, int32_t* bad);
-// degree statistics: the row lengths of `off`, plus those of `off2` when it is not null
-__global__ void k_deg_reduce(const int32_t* off, const int32_t* off2, int32_t n, unsigned long long* s1,
-                             unsigned long long* s2, unsigned int* dmin, unsigned int* dmax);
-__global__ void k_deg_hist(const int32_t* off, const int32_t* off2, int32_t n, int32_t* hist);
-__global__ void k_deg_finish(const int32_t* hist, int64_t maxdeg, int32_t n, const unsigned long long* s1,
-                             const unsigned long long* s2, long long* out6);
+// degree statistics: out-, in- and total degree (in null: a symmetric graph, out-degree only)
+struct DegSums {
+  unsigned long long s1, s2;
+  unsigned int dmax, pad;
+};
+constexpr int kDegFinishThreads = 1024;
+__global__ void k_deg_reduce(const int32_t* off, const int32_t* off_in, int32_t n, DegSums* out);
+__global__ void k_deg_hist(const int32_t* off, const int32_t* off_in, int32_t n, long long at1, long long at2,
+                           int32_t* hist);
+__global__ void k_deg_finish(const int32_t* hist, long long at1, long long at2, int32_t n, const DegSums* sums,
+                             int32_t symmetric, long long* out);
 __global__ void k_tr_count(const int32_t* idx, int32_t m, int32_t* cnt);
 __global__ void k_scan_reduce(const int32_t* in, int32_t len, long long* bsum);
 __global__ void k_scan_top(long long* bsum, int32_t nblocks);
 __global__ void k_scan_apply(const int32_t* in, int32_t len, const long long* bsum, int32_t* out);
-__global__ void k_tr_scatter(const int32_t* off, const int32_t* idx, int32_t n, int32_t* cursor, int32_t* in_idx);
+__global__ void k_tr_scatter(const int32_t* off, const int32_t* idx, int32_t n, int32_t m, int32_t* cursor,
+                             int32_t* in_idx);
 __global__ void k_records(const int32_t* off, const int32_t* idx, int32_t n, int32_t w, int32_t* rec);
 __global__ void k_pull_hint(const int32_t* off, const int32_t* in_off, const int32_t* in_idx, int32_t n,
                             int32_t* hint);
