@@ -242,9 +242,26 @@ struct bfs_graph {
   MsConfig ms_cfg{0, 16};
   int ms_grid = 0;       // one full occupancy wave of the multi-source kernel
   int ms_grid_user = 0;  // configured grid (0: ms_grid)
+  cudaStream_t upload = nullptr;  // small synchronous copies to the device (upload_now)
 };
 
 namespace {
+
+// Parts of one device allocation: add() each part's bytes first (offsets are
+// multiples of 256 bytes, as cudaMalloc's addresses are), then allocate size().
+struct Arena {
+  size_t size_ = 0;
+  size_t add(size_t bytes) {
+    const size_t at = size_;
+    size_ += (std::max<size_t>(bytes, 1) + 255) & ~size_t(255);
+    return at;
+  }
+  size_t size() const { return size_; }
+  template <typename T>
+  static T* at(void* base, size_t offset) {
+    return reinterpret_cast<T*>(static_cast<char*>(base) + offset);
+  }
+};
 
 int grid_for(const void* func, int sms, int cap_per_sm) {
   int per_sm = 0;
@@ -260,13 +277,11 @@ int grid_for(const void* func, int sms, int cap_per_sm) {
 // cudaMemcpy from pageable memory may return once the source is staged, before
 // its DMA lands, and a kernel launched next on a non-blocking stream is not
 // ordered after that DMA: it could read the old contents, or have its own
-// writes overwritten when the DMA lands.
-int upload_now(void* dst, const void* src, size_t bytes) {
-  cudaStream_t s;
-  CU(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
-  cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  cudaStreamDestroy(s);
+// writes overwritten when the DMA lands. The copy goes through the graph's own
+// non-blocking stream, so it waits for no run of the caller's.
+int upload_now(const bfs_graph* g, void* dst, const void* src, size_t bytes) {
+  cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, g->upload);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(g->upload);
   if (e != cudaSuccess) return fail(BFS_ERR_CUDA, "upload of %zu bytes: %s", bytes, cudaGetErrorString(e));
   return BFS_OK;
 }
@@ -311,7 +326,7 @@ int add_kernel(cudaGraph_t graph, cudaGraphNode_t* node, const cudaGraphNode_t* 
 
 // The workspace's device state before its first run: the log buffers and, once
 // the level-loop graph exists, its conditional handles.
-int init_run_state(Workspace* ws, unsigned long long h_while, unsigned long long h_switch) {
+int init_run_state(const bfs_graph* g, Workspace* ws, unsigned long long h_while, unsigned long long h_switch) {
   RunState init{};
   init.h_while = h_while;
   init.h_switch = h_switch;
@@ -321,7 +336,7 @@ int init_run_state(Workspace* ws, unsigned long long h_while, unsigned long long
   init.log_frontier = ws->log_frontier;
   init.log_edges = ws->log_edges;
   init.log_time = ws->log_time;
-  return upload_now(ws->st, &init, sizeof init);
+  return upload_now(g, ws->st, &init, sizeof init);
 }
 
 // Build the level loop of one workspace as a CUDA graph with conditional nodes
@@ -388,37 +403,38 @@ int build_graph(bfs_graph* g, Workspace* ws) {
                  kThreads, ka));
   CU(cudaGraphInstantiate(&ws->exec, ws->graph, 0));
   // the handles live in the device state, where decide sets them each level
-  return init_run_state(ws, hw, hs);
+  return init_run_state(g, ws, hw, hs);
 }
 
 int create_workspace(bfs_graph* g, Workspace** out) {
   auto* ws = new Workspace;
-  const int64_t n = g->dg.n;
-  const int64_t words = g->dg.words;
-  int r = BFS_OK;
-  void* p;
-  auto A = [&](size_t bytes) -> void* {
-    if (r != BFS_OK) return nullptr;
-    r = ws_alloc(ws, &p, bytes);
-    return r == BFS_OK ? p : nullptr;
-  };
-  ws->b.q[0] = static_cast<int32_t*>(A(n * 4));
-  ws->b.q[1] = static_cast<int32_t*>(A(n * 4));
-  ws->b.vis[0] = static_cast<uint32_t*>(A(words * 4));
-  ws->b.vis[1] = static_cast<uint32_t*>(A(words * 4));
-  ws->b.heavy_cap = (int32_t)std::min<int64_t>(n, kHeavyCap);
-  ws->b.heavy = static_cast<int32_t*>(A((size_t)ws->b.heavy_cap * 4));
-  ws->st = static_cast<RunState*>(A(sizeof(RunState)));
-  ws->log_cap = (int32_t)std::min<int64_t>(n + 1, 1 << 16);
-  ws->log_variant = static_cast<int32_t*>(A(ws->log_cap * 4));
-  ws->log_frontier = static_cast<long long*>(A(ws->log_cap * 8));
-  ws->log_edges = static_cast<long long*>(A(ws->log_cap * 8));
-  ws->log_time = static_cast<long long*>(A(ws->log_cap * 8));
+  const size_t n = (size_t)g->dg.n, words = (size_t)g->dg.words;
+  ws->b.heavy_cap = (int32_t)std::min<size_t>(n, kHeavyCap);
+  ws->log_cap = (int32_t)std::min<size_t>(n + 1, 1 << 16);
+  const size_t log = (size_t)ws->log_cap;
+  Arena a;
+  const size_t q0 = a.add(n * 4), q1 = a.add(n * 4), v0 = a.add(words * 4), v1 = a.add(words * 4),
+               heavy = a.add((size_t)ws->b.heavy_cap * 4), st = a.add(sizeof(RunState)), lv = a.add(log * 4),
+               lf = a.add(log * 8), le = a.add(log * 8), lt = a.add(log * 8);
+  void* p = nullptr;
+  int r = ws_alloc(ws, &p, a.size());
+  if (r == BFS_OK) {
+    ws->b.q[0] = Arena::at<int32_t>(p, q0);
+    ws->b.q[1] = Arena::at<int32_t>(p, q1);
+    ws->b.vis[0] = Arena::at<uint32_t>(p, v0);
+    ws->b.vis[1] = Arena::at<uint32_t>(p, v1);
+    ws->b.heavy = Arena::at<int32_t>(p, heavy);
+    ws->st = Arena::at<RunState>(p, st);
+    ws->log_variant = Arena::at<int32_t>(p, lv);
+    ws->log_frontier = Arena::at<long long>(p, lf);
+    ws->log_edges = Arena::at<long long>(p, le);
+    ws->log_time = Arena::at<long long>(p, lt);
+  }
   if (r == BFS_OK) {
     cudaError_t e = cudaEventCreateWithFlags(&ws->done, cudaEventDisableTiming);
     if (e != cudaSuccess) r = fail(BFS_ERR_CUDA, "cudaEventCreate: %s", cudaGetErrorString(e));
   }
-  if (r == BFS_OK) r = init_run_state(ws, 0, 0);
+  if (r == BFS_OK) r = init_run_state(g, ws, 0, 0);
   if (r != BFS_OK) {
     free_workspace(ws);
     return r;
@@ -654,7 +670,7 @@ int sync_tree(bfs_graph* g) {
   if (has_qs) std::memcpy(host.data() + qs_off, &qs, sizeof qs);
   void* p = nullptr;
   TRY(dmalloc(&p, host.size()));
-  const int r = upload_now(p, host.data(), host.size());
+  const int r = upload_now(g, p, host.data(), host.size());
   if (r != BFS_OK) {
     cudaFree(p);
     return r;
@@ -696,7 +712,7 @@ int ensure_origin(bfs_graph* g) {
   cudaStreamDestroy(s);
   if (e != cudaSuccess) return fail(BFS_ERR_CUDA, "origin arrays: %s", cudaGetErrorString(e));
   const GraphAux aux{out, in};
-  TRY(upload_now(g->aux, &aux, sizeof aux));
+  TRY(upload_now(g, g->aux, &aux, sizeof aux));
   g->has_origin = true;
   return BFS_OK;
 }
@@ -977,7 +993,7 @@ int bfs::ms_set_create(bfs_graph* g, MsSet** out) {
   }
   if (r == BFS_OK) {
     MsState init{};  // clean_blocks == clean_grid: the masks are zero
-    r = upload_now(set->st, &init, sizeof init);
+    r = upload_now(g, set->st, &init, sizeof init);
   }
   if (r != BFS_OK) {
     ms_set_free(set);
@@ -1017,49 +1033,6 @@ int bfs::batch_async(bfs_graph* g, MsSet* set, const int32_t* roots, int32_t k, 
 }
 
 namespace {
-
-// The 5-number summaries (nearest rank) and floor(256 sd) of the out-, in- and
-// total degrees of all n vertices, on the device: the row lengths of `off`, of
-// `off_in` (null: a symmetric graph) and their sums. Synchronous.
-int degree_summaries(const int32_t* off, const int32_t* off_in, int32_t n, int blocks, long long out6[6],
-                     long long in6[6], long long tot6[6]) {
-  struct Block {
-    DegSums sums[3];
-    long long out[18];
-  };
-  Block* d = nullptr;
-  Block h{};
-  int32_t* hist = nullptr;
-  cudaError_t e = cudaMalloc(&d, sizeof(Block));
-  if (e == cudaSuccess) e = cudaMemset(d, 0, sizeof(Block));
-  if (e == cudaSuccess) {
-    k_deg_reduce<<<blocks, kThreads>>>(off, off_in, n, d->sums);
-    e = cudaMemcpy(&h, d, sizeof h.sums, cudaMemcpyDeviceToHost);
-  }
-  // the kinds' histograms one after another
-  const long long at1 = (long long)h.sums[0].dmax + 1, at2 = at1 + (long long)h.sums[1].dmax + 1;
-  const size_t bins = (size_t)(off_in ? at2 + (long long)h.sums[2].dmax + 1 : at1);
-  if (e == cudaSuccess) e = cudaMalloc(&hist, bins * 4);
-  if (e == cudaSuccess) e = cudaMemset(hist, 0, bins * 4);
-  if (e == cudaSuccess) {
-    k_deg_hist<<<blocks, kThreads>>>(off, off_in, n, at1, at2, hist);
-    k_deg_finish<<<off_in ? 3 : 2, kDegFinishThreads>>>(hist, at1, at2, n, d->sums, off_in ? 0 : 1, d->out);
-    e = cudaMemcpy(h.out, d->out, sizeof h.out, cudaMemcpyDeviceToHost);
-  }
-  if (d) cudaFree(d);
-  if (hist) cudaFree(hist);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return fail(e == cudaErrorMemoryAllocation ? BFS_ERR_OOM : BFS_ERR_CUDA, "degree statistics: %s",
-                cudaGetErrorString(e));
-  }
-  for (int k = 0; k < 6; ++k) {
-    out6[k] = h.out[k];
-    in6[k] = off_in ? h.out[6 + k] : h.out[k];
-    tot6[k] = off_in ? h.out[12 + k] : h.out[6 + k];
-  }
-  return BFS_OK;
-}
 
 // The tree's choice for a level on the host (the same walk and unknown-
 // prediction rule the device applies): features are exact integers, so every
@@ -1234,9 +1207,13 @@ int bfs_graph_create(const int32_t* row_offsets, const int32_t* col_indices, int
   CU(cudaGetDevice(&g->device));
   CU(cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, g->device));
   g->symmetric = (flags & BFS_SYMMETRIC) != 0;
+  void* temp = nullptr;  // what only this call needs
   auto cleanup = [&]() {
     for (void* p : g->allocs) cudaFree(p);
     g->allocs.clear();
+    if (temp) cudaFree(temp);
+    if (g->upload) cudaStreamDestroy(g->upload);
+    cudaGetLastError();
   };
   auto galloc = [&](void** p, size_t bytes) -> int {
     int r = dmalloc(p, bytes);
@@ -1247,119 +1224,111 @@ int bfs_graph_create(const int32_t* row_offsets, const int32_t* col_indices, int
     return r;
   };
   const cudaMemcpyKind kind = (flags & BFS_INPUT_ON_DEVICE) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-  int32_t *off = nullptr, *idx = nullptr;
-  int r = galloc(reinterpret_cast<void**>(&off), (n + 1) * 4);
-  if (r == BFS_OK) r = galloc(reinterpret_cast<void**>(&idx), (m + kIdxPad) * 4);
-  if (r != BFS_OK) {
+  const int64_t words = (n + 31) / 32;
+  const int64_t nblk = (n + kPeTile - 1) / kPeTile;
+  // the graph's arrays in one allocation: the CSR, its transpose for pull when
+  // the graph may be directed, the starting bitmap, the edge-list variants'
+  // pointers and the pull hints
+  Arena ga;
+  const size_t a_off = ga.add((size_t)(n + 1) * 4), a_idx = ga.add((size_t)(m + kIdxPad) * 4);
+  const size_t a_in_off = g->symmetric ? a_off : ga.add((size_t)(n + 1) * 4);
+  const size_t a_in_idx = g->symmetric ? a_idx : ga.add((size_t)(m + kIdxPad) * 4);
+  const size_t a_vis = ga.add((size_t)words * 4), a_aux = ga.add(sizeof(GraphAux)), a_hint = ga.add((size_t)n * 4);
+  struct Found {  // what the checks and statistics report
+    int32_t bad;
+    unsigned int isolated;
+    DegSums sums[3];
+    long long out[18];
+  };
+  Arena ta;
+  const size_t t_found = ta.add(sizeof(Found));
+  const size_t t_cnt = g->symmetric ? 0 : ta.add((size_t)(n + 1) * 4), t_bsum = g->symmetric ? 0 : ta.add((size_t)(nblk + 2) * 8);
+  void* base = nullptr;
+  int r = galloc(&base, ga.size());
+  cudaError_t e = cudaSuccess;
+  if (r == BFS_OK) e = cudaMalloc(&temp, ta.size());
+  if (r == BFS_OK && e == cudaSuccess) e = cudaStreamCreateWithFlags(&g->upload, cudaStreamNonBlocking);
+  if (r != BFS_OK || e != cudaSuccess) {
     cleanup();
-    return r;
+    return r != BFS_OK ? r : fail(e == cudaErrorMemoryAllocation ? BFS_ERR_OOM : BFS_ERR_CUDA, "graph create: %s",
+                                  cudaGetErrorString(e));
   }
-  cudaError_t e = cudaMemcpy(off, row_offsets, (n + 1) * 4, kind);
-  if (e == cudaSuccess && m > 0) e = cudaMemcpy(idx, col_indices, m * 4, kind);
-  if (e == cudaSuccess) e = cudaMemset(idx + m, 0, kIdxPad * 4);
-  // validation is unconditional: a malformed CSR would make kernels read out of bounds
-  int32_t* scratch = nullptr;  // [0] bad flag, [1] dmin, [2] dmax
-  unsigned long long* sums = nullptr;
-  if (e == cudaSuccess) e = cudaMalloc(&scratch, 16);
-  if (e == cudaSuccess) e = cudaMalloc(&sums, 16);
-  if (e != cudaSuccess) {
-    if (scratch) cudaFree(scratch);
-    cleanup();
-    return fail(BFS_ERR_CUDA, "graph upload: %s", cudaGetErrorString(e));
-  }
+  int32_t* const off = Arena::at<int32_t>(base, a_off);
+  int32_t* const idx = Arena::at<int32_t>(base, a_idx);
+  int32_t* const in_off = Arena::at<int32_t>(base, a_in_off);
+  int32_t* const in_idx = Arena::at<int32_t>(base, a_in_idx);
+  uint32_t* const vis_init = Arena::at<uint32_t>(base, a_vis);
+  int32_t* const hint = Arena::at<int32_t>(base, a_hint);
+  g->aux = Arena::at<GraphAux>(base, a_aux);
+  Found* const found = Arena::at<Found>(temp, t_found);
+  Found h{};
   const int blocks = g->sms * 4;
-  int32_t init3[3] = {0, INT32_MAX, 0};
-  cudaMemcpy(scratch, init3, 12, cudaMemcpyHostToDevice);
-  cudaMemset(sums, 0, 16);
-  k_validate<<<blocks, kThreads>>>(off, idx, (int32_t)n, (int32_t)m, scratch);
-  int32_t bad = 0;
-  e = cudaMemcpy(&bad, scratch, 4, cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess || bad) {
-    cudaFree(scratch);
-    cudaFree(sums);
+  e = cudaMemcpy(off, row_offsets, (n + 1) * 4, kind);
+  if (e == cudaSuccess && m > 0) e = cudaMemcpy(idx, col_indices, m * 4, kind);
+  if (e == cudaSuccess) e = cudaMemsetAsync(idx + m, 0, kIdxPad * 4);
+  if (e == cudaSuccess) e = cudaMemsetAsync(g->aux, 0, sizeof(GraphAux));
+  if (e == cudaSuccess) e = cudaMemsetAsync(found, 0, sizeof(Found));
+  // validation is unconditional: a malformed CSR would make kernels read out of bounds
+  if (e == cudaSuccess) {
+    k_validate<<<blocks, kThreads>>>(off, idx, (int32_t)n, (int32_t)m, &found->bad);
+    e = cudaMemcpy(&h.bad, &found->bad, sizeof h.bad, cudaMemcpyDeviceToHost);
+  }
+  if (e != cudaSuccess || h.bad) {
     cleanup();
     if (e != cudaSuccess) return fail(BFS_ERR_CUDA, "validate: %s", cudaGetErrorString(e));
     return fail(BFS_ERR_BAD_GRAPH, "CSR failed validation (off[0]=0, nondecreasing, off[n]=m, 0<=idx<n)");
   }
-  cudaFree(scratch);
-  cudaFree(sums);
-  // transpose for pull when the graph may be directed
-  int32_t *in_off = off, *in_idx = idx;
   if (!g->symmetric) {
-    r = galloc(reinterpret_cast<void**>(&in_off), (n + 1) * 4);
-    if (r == BFS_OK) r = galloc(reinterpret_cast<void**>(&in_idx), (m + kIdxPad) * 4);
-    int32_t* cnt = nullptr;
-    long long* bsum = nullptr;
-    const int64_t nblk = (n + kPeTile - 1) / kPeTile;
-    if (r == BFS_OK) {
-      e = cudaMalloc(&cnt, (n + 1) * 4);
-      if (e == cudaSuccess) e = cudaMalloc(&bsum, (nblk + 2) * 8);
-      if (e == cudaSuccess) e = cudaMemset(cnt, 0, (n + 1) * 4);
-      if (e == cudaSuccess) e = cudaMemset(in_idx + m, 0, kIdxPad * 4);
-      if (e == cudaSuccess) {
-        k_tr_count<<<blocks, kThreads>>>(idx, (int32_t)m, cnt);
-        k_scan_reduce<<<blocks, kThreads>>>(cnt, (int32_t)n, bsum);
-        k_scan_top<<<1, kThreads>>>(bsum, (int32_t)nblk);
-        k_scan_apply<<<blocks, kThreads>>>(cnt, (int32_t)n, bsum, in_off);
-        e = cudaMemcpy(cnt, in_off, (n + 1) * 4, cudaMemcpyDeviceToDevice);
-      }
-      if (e == cudaSuccess) {
-        k_tr_scatter<<<g->sms * 8, kThreads>>>(off, idx, (int32_t)n, (int32_t)m, cnt, in_idx);
-        e = cudaDeviceSynchronize();
-      }
-      if (e != cudaSuccess) r = fail(BFS_ERR_CUDA, "transpose: %s", cudaGetErrorString(e));
+    int32_t* const cnt = Arena::at<int32_t>(temp, t_cnt);
+    long long* const bsum = Arena::at<long long>(temp, t_bsum);
+    e = cudaMemsetAsync(cnt, 0, (n + 1) * 4);
+    if (e == cudaSuccess) e = cudaMemsetAsync(in_idx + m, 0, kIdxPad * 4);
+    if (e == cudaSuccess) {
+      k_tr_count<<<blocks, kThreads>>>(idx, (int32_t)m, cnt);
+      k_scan_reduce<<<blocks, kThreads>>>(cnt, (int32_t)n, bsum);
+      k_scan_top<<<1, kThreads>>>(bsum, (int32_t)nblk);
+      k_scan_apply<<<blocks, kThreads>>>(cnt, (int32_t)n, bsum, in_off);
+      e = cudaMemcpyAsync(cnt, in_off, (n + 1) * 4, cudaMemcpyDeviceToDevice);
     }
-    if (cnt) cudaFree(cnt);
-    if (bsum) cudaFree(bsum);
-    if (r != BFS_OK) {
-      cleanup();
-      return r;
-    }
+    if (e == cudaSuccess) k_tr_scatter<<<g->sms * 8, kThreads>>>(off, idx, (int32_t)n, (int32_t)m, cnt, in_idx);
   }
-  // starting bitmap: isolated vertices are marked visited up front
-  uint32_t* vis_init = nullptr;
-  const int64_t words = (n + 31) / 32;
-  r = galloc(reinterpret_cast<void**>(&vis_init), words * 4);
-  if (r == BFS_OK) r = galloc(reinterpret_cast<void**>(&g->aux), sizeof(GraphAux));
-  if (r == BFS_OK) {
-    const GraphAux none{nullptr, nullptr};
-    r = upload_now(g->aux, &none, sizeof none);
-  }
-  if (r != BFS_OK) {
-    cleanup();
-    return r;
-  }
-  // the pull variant's first test per vertex (k_pull_hint)
-  int32_t* hint = nullptr;
-  r = galloc(reinterpret_cast<void**>(&hint), (size_t)n * 4);
-  if (r != BFS_OK) {
-    cleanup();
-    return r;
-  }
-  k_pull_hint<<<blocks, kThreads>>>(off, in_off, in_idx, (int32_t)n, hint);
-  unsigned int* iso = nullptr;
-  unsigned int iso_h = 0;
-  e = cudaMalloc(&iso, sizeof(unsigned int));
-  if (e == cudaSuccess) e = cudaMemset(iso, 0, sizeof(unsigned int));
+  // the pull variant's first test per vertex; the starting bitmap, isolated
+  // vertices marked visited up front; the degree sums and maxima
+  const int32_t* const deg_in = g->symmetric ? nullptr : in_off;
   if (e == cudaSuccess) {
-    k_vis_init<<<blocks, kThreads>>>(off, in_off, (int32_t)n, (int32_t)words, vis_init, iso);
-    e = cudaDeviceSynchronize();
+    k_pull_hint<<<blocks, kThreads>>>(off, in_off, in_idx, (int32_t)n, hint);
+    k_vis_init<<<blocks, kThreads>>>(off, in_off, (int32_t)n, (int32_t)words, vis_init, &found->isolated);
+    k_deg_reduce<<<blocks, kThreads>>>(off, deg_in, (int32_t)n, found->sums);
+    e = cudaMemcpy(&h, found, sizeof h, cudaMemcpyDeviceToHost);
   }
-  if (e == cudaSuccess) e = cudaMemcpy(&iso_h, iso, sizeof iso_h, cudaMemcpyDeviceToHost);
-  if (iso) cudaFree(iso);
+  // degree summaries (Section 4.1 degree distribution): out-degree, in-degree
+  // (the transpose's row lengths) and total degree, from their histograms, one
+  // after another in one allocation
+  const long long at1 = (long long)h.sums[0].dmax + 1, at2 = at1 + (long long)h.sums[1].dmax + 1;
+  const size_t bins = (size_t)(deg_in ? at2 + (long long)h.sums[2].dmax + 1 : at1);
+  int32_t* hist = nullptr;
+  if (e == cudaSuccess) e = cudaMalloc(&hist, bins * 4);
+  if (e == cudaSuccess) e = cudaMemsetAsync(hist, 0, bins * 4);
+  if (e == cudaSuccess) {
+    k_deg_hist<<<blocks, kThreads>>>(off, deg_in, (int32_t)n, at1, at2, hist);
+    k_deg_finish<<<deg_in ? 3 : 2, kDegFinishThreads>>>(hist, at1, at2, (int32_t)n, found->sums, deg_in ? 0 : 1,
+                                                        found->out);
+    e = cudaMemcpy(h.out, found->out, sizeof h.out, cudaMemcpyDeviceToHost);
+  }
+  if (hist) cudaFree(hist);
   if (e != cudaSuccess) {
     cleanup();
     return fail(e == cudaErrorMemoryAllocation ? BFS_ERR_OOM : BFS_ERR_CUDA, "graph create: %s",
                 cudaGetErrorString(e));
   }
-  // degree statistics (Section 4.1 degree distribution): out-degree, in-degree
-  // (the transpose's row lengths) and total degree
-  r = degree_summaries(off, g->symmetric ? nullptr : in_off, (int32_t)n, blocks, g->stats6, g->stats_in6,
-                       g->stats_tot6);
-  if (r != BFS_OK) {
-    cleanup();
-    return r;
+  for (int k = 0; k < 6; ++k) {
+    g->stats6[k] = h.out[k];
+    g->stats_in6[k] = deg_in ? h.out[6 + k] : h.out[k];
+    g->stats_tot6[k] = deg_in ? h.out[12 + k] : h.out[6 + k];
   }
+  const unsigned int iso_h = h.isolated;
+  cudaFree(temp);
+  temp = nullptr;
   // vertex records where every list is short (k_records); a graph they do not
   // fit beside is used without
   int32_t* rec = nullptr;
@@ -1391,7 +1360,7 @@ int bfs_graph_create(const int32_t* row_offsets, const int32_t* col_indices, int
   dg.aux = g->aux;
   dg.n = (int32_t)n;
   dg.m = (int32_t)m;
-  dg.words = (int32_t)((n + 31) / 32);
+  dg.words = (int32_t)words;
   dg.symmetric = g->symmetric ? 1 : 0;
   dg.n_active = (int32_t)(n - (int64_t)iso_h);
   dg.gfeat[F_N] = n;
@@ -1463,6 +1432,7 @@ int bfs_graph_destroy(bfs_graph_t g) {
   for (TreeNode* t : g->trees) cudaFree(t);
   bfs::ms_set_free(g->ms_set);
   for (void* p : g->allocs) cudaFree(p);
+  if (g->upload) cudaStreamDestroy(g->upload);
   delete g;
   if (e != cudaSuccess) return fail(BFS_ERR_CUDA, "destroy: %s", cudaGetErrorString(e));
   return BFS_OK;
