@@ -290,11 +290,12 @@ int bfs_run_batch(bfs_graph_t g, const int32_t* roots, int32_t k, int32_t* depth
 
 /* Launch shape of the multi-source kernel (chosen by bfs_batch_tune). */
 typedef struct bfs_batch_config {
-  int32_t push_mode;  /* 0: one thread per frontier vertex, 1: one warp per frontier vertex */
+  int32_t push_mode;  /* 0: a block's frontier vertices' edges dealt to its threads, 1: one warp per
+                         frontier vertex */
   int32_t alpha;      /* a level pulls when its frontier's edge count x alpha exceeds m */
   float ms;           /* bfs_batch_tune: measured time of one wave with this configuration */
   int32_t grid_blocks; /* blocks of the multi-source kernel (larger values are clamped to one full
-                          occupancy wave); 0 for a grid sized to the graph: one block per 4096
+                          occupancy wave); 0 for a grid sized to the graph: one block per 1024
                           vertices, at least a quarter of the SMs, at most one full occupancy
                           wave (so that small graphs' waves on several streams run together) */
 } bfs_batch_config;

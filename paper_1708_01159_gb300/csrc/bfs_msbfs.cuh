@@ -33,6 +33,7 @@ struct MsState {
   unsigned int ftail[4];           // frontier list length (= frontier vertices) of level L in slot L % 4
   unsigned int ttail[2];           // touched list length of a push level L in slot L % 2
   unsigned long long fedges[4];    // out-degree sum of level L's frontier, slot L % 4
+  unsigned long long alive[4];     // roots with a vertex in level L's frontier, slot L % 4
   unsigned long long edges[kMsMaxRoots];  // reached-edge count per root
   // Between waves the history arrays are all zero when clean_blocks ==
   // clean_grid: every block of the last wave cleared what the wave set (the
@@ -43,7 +44,7 @@ struct MsState {
 };
 
 struct MsConfig {
-  int32_t push_mode;  // 0: thread per frontier vertex, 1: warp per frontier vertex
+  int32_t push_mode;  // 0: a block's frontier vertices' edges dealt to its threads, 1: warp per frontier vertex
   int32_t alpha;      // a level pulls when its frontier edges x alpha exceed m
 };
 
