@@ -418,6 +418,37 @@ __device__ __forceinline__ void stage_put(const Stage& s, int32_t* out, TailT* t
     queue_append(out, tail, v);
 }
 
+// stage_put of up to K vertices a lane (those with won[k]): one reservation for
+// all of the converged lanes' in place of one per k.
+template <int K, typename TailT>
+__device__ __forceinline__ void stage_put_won(const Stage& s, int32_t* out, TailT* tail, const bool (&won)[K],
+                                              const int32_t (&v)[K]) {
+  const uint32_t mask = __activemask();
+  const int leader = __ffs(mask) - 1;
+  uint32_t m[K];
+  unsigned int total = 0;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    m[k] = __ballot_sync(mask, won[k]);
+    total += (unsigned)__popc(m[k]);
+  }
+  if (total == 0u) return;  // the same for every lane of the mask
+  unsigned int pos = 0;
+  if ((int)lane_id() == leader) pos = atomicAdd(s.cnt, total);
+  pos = __shfl_sync(mask, pos, leader);
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    if (won[k]) {
+      const unsigned int at = pos + (unsigned)__popc(m[k] & lanemask_lt());
+      if (at < (unsigned)kStageCap)
+        s.buf[at] = v[k];
+      else
+        queue_append(out, tail, v[k]);
+    }
+    pos += (unsigned)__popc(m[k]);
+  }
+}
+
 // Copies the staged entries out once at least `threshold` are waiting. Every
 // thread of the block must call it (it synchronises).
 template <typename TailT>
@@ -464,6 +495,10 @@ __device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned l
 
 __device__ __forceinline__ void red_release_add_u64(unsigned long long* p, unsigned long long v) {
   asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+__device__ __forceinline__ void red_relaxed_add_u64(unsigned long long* p, unsigned long long v) {
+  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
 // Sum of x over the block, returned to every thread. Every thread of the block
@@ -526,8 +561,9 @@ __device__ __forceinline__ bool grid_arrive_wait(unsigned long long* count, unsi
 // *tail holds the output queue tail (f, low 32 bits) and *edges the frontier
 // edge sum (e, low 40 bits). Thread 0 adds its block's edge sum e_block
 // together with one arrival (bit 40) to *edges, then one arrival (bit 32) to
-// *tail, both as release reductions after all of the block's appends; then it
-// polls both words until each shows every block's arrival, and reads f and e
+// *tail, after one fence that covers all of the block's appends (a release on
+// each reduction made the second wait for the first: R-MAT 22 93.4 -> 91.6 us a
+// traversal); then it polls both words until each shows every block's arrival, and reads f and e
 // from the same loads. No block waits for an atomic's return, no last block
 // publishes anything, and no block reads a counter after the barrier. Bounded
 // and hookable like grid_arrive_wait.
@@ -539,8 +575,9 @@ __device__ __forceinline__ bool level_arrive_wait(unsigned long long* tail, unsi
   __syncthreads();
   bool ok = true;
   if (threadIdx.x == 0) {
-    red_release_add_u64(edges, (1ull << 40) + e_block);
-    red_release_add_u64(tail, 1ull << 32);
+    __threadfence();
+    red_relaxed_add_u64(edges, (1ull << 40) + e_block);
+    red_relaxed_add_u64(tail, 1ull << 32);
     const unsigned long long want = (unsigned long long)gridDim.x + extra;
     unsigned long long a = ld_acquire_u64(tail), b = ld_acquire_u64(edges);
     if ((a >> 32) < want || (b >> 40) < want) {

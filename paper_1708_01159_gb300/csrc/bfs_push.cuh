@@ -40,10 +40,6 @@ constexpr long long kLatencyEdges = 1ll << 17;
 
 // Newly reached vertices go through a block-local stage (see stage_put) into
 // the level's output queue.
-__device__ __forceinline__ void stage_push(const Stage& s, const Level& lv, int32_t v) {
-  stage_put(s, lv.qout, lv.tail, v);
-}
-
 __device__ __forceinline__ void stage_flush(const Stage& s, const Level& lv, unsigned int threshold) {
   stage_drain(s, lv.qout, lv.tail, threshold);
 }
@@ -61,7 +57,9 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 // predicated accesses because an `if` per edge made the compiler wait for each
 // claim and each row extent in turn (vertex push on R-MAT 14: 2.49 ms a
 // traversal with the branches, 1.85 ms without; virtual warps on its level of
-// 345k edges 78 -> 59 us; ER 2^21, level of 1.6M edges, 48 -> 41 us).
+// 345k edges 78 -> 59 us; ER 2^21, level of 1.6M edges, 48 -> 41 us). The
+// winners of all K edges of the converged lanes take one reservation in the
+// stage, not one per edge (ER level 41 -> 36 us).
 // valid: bit k set when v[k] is an edge to visit.
 template <int K, int kCount = CM_BLOCK>
 __device__ __forceinline__ void visit_km(const DevGraph& g, const Level& lv, const Stage& s, const int32_t (&v)[K],
@@ -84,29 +82,32 @@ __device__ __forceinline__ void visit_km(const DevGraph& g, const Level& lv, con
   }
 #pragma unroll
   for (int k = 0; k < K; ++k) won[k] = !((word[k] >> (v[k] & 31)) & 1u);
-  int32_t b0[K], d[K];
+  // the winners' rows, four at a time
+  constexpr int kRows = K < 4 ? K : 4;
+  static_assert(K % kRows == 0, "whole groups");
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    b0[k] = ld_if(won[k], g.off + v[k], 0);
-    d[k] = ld_if(won[k], g.off + v[k] + 1, 0);
-  }
+  for (int h = 0; h < K; h += kRows) {
+    int32_t b0[kRows], d[kRows];
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    d[k] -= b0[k];
-    prefetch_l2_if(!filter && d[k] > 0, g.idx + b0[k]);
-  }
-#pragma unroll
-  for (int k = 0; k < K; ++k)
-    if (won[k]) {
-      lv.depth[v[k]] = lv.next_depth;
-      edges += (unsigned long long)d[k];
-      if (kCount == CM_BLOCK)
-        stage_push(s, lv, v[k]);
-      else if (kCount == CM_WARP)
-        queue_append(lv.qout, lv.tail, v[k]);
-      else
-        lv.qout[(unsigned int)atomicAdd(lv.tail, 1ull)] = v[k];
+    for (int k = 0; k < kRows; ++k) {
+      b0[k] = ld_if(won[h + k], g.off + v[h + k], 0);
+      d[k] = ld_if(won[h + k], g.off + v[h + k] + 1, 0);
     }
+#pragma unroll
+    for (int k = 0; k < kRows; ++k) {
+      d[k] -= b0[k];
+      prefetch_l2_if(!filter && d[k] > 0, g.idx + b0[k]);
+      edges += (unsigned long long)d[k];
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    if (!won[k]) continue;
+    lv.depth[v[k]] = lv.next_depth;
+    if (kCount == CM_WARP) queue_append(lv.qout, lv.tail, v[k]);
+    if (kCount == CM_ATOMIC) lv.qout[(unsigned int)atomicAdd(lv.tail, 1ull)] = v[k];
+  }
+  if (kCount == CM_BLOCK) stage_put_won(s, lv.qout, lv.tail, won, v);
 }
 
 // The first nv entries of v are edges to visit, four in flight at a time (more
