@@ -99,6 +99,67 @@ TRAIN_GRAPHS = [
     ("rmat", dict(scale=20, edge_factor=8, seed=3025, directed=True, b=0.08, c=0.30)),
     ("rmat", dict(scale=21, edge_factor=16, seed=3026, directed=True)),
     ("rmat", dict(scale=22, edge_factor=8, seed=3027, directed=True, b=0.25, c=0.13)),
+    # small graphs, where the launch-bound levels and the few wide ones trade places
+    ("rmat", dict(scale=12, edge_factor=16, seed=3028)),
+    ("rmat", dict(scale=13, edge_factor=8, seed=3029)),
+    ("rmat", dict(scale=14, edge_factor=16, seed=3030)),
+    ("rmat", dict(scale=14, edge_factor=32, seed=3031, permute=True)),
+    ("rmat", dict(scale=15, edge_factor=24, seed=3032)),
+    ("rmat", dict(scale=13, edge_factor=16, seed=3033, directed=True, b=0.25, c=0.13)),
+    ("rmat", dict(scale=17, edge_factor=16, seed=3034, directed=True)),
+    ("rmat", dict(scale=19, edge_factor=16, seed=3035, directed=True)),
+    ("rmat", dict(scale=20, edge_factor=16, seed=3036, directed=True)),
+    ("er", dict(n=6000, avg_degree=16.0, seed=3037)),
+    ("er", dict(n=1 << 14, avg_degree=8.0, seed=3038)),
+    ("er", dict(n=1 << 16, avg_degree=24.0, seed=3039)),
+    ("er", dict(n=200000, avg_degree=4.0, seed=3040)),
+    ("er", dict(n=700000, avg_degree=16.0, seed=3041)),
+    ("grid", dict(rows=64, cols=200, drop=0.1, seed=3042)),
+    ("er", dict(n=4096, avg_degree=4.0, seed=3043)),
+    ("er", dict(n=8192, avg_degree=8.0, seed=3044)),
+    ("er", dict(n=10000, avg_degree=32.0, seed=3045)),
+    ("er", dict(n=30000, avg_degree=16.0, seed=3046)),
+    ("er", dict(n=50000, avg_degree=8.0, seed=3047)),
+    ("er", dict(n=120000, avg_degree=24.0, seed=3048)),
+    ("er", dict(n=400000, avg_degree=8.0, seed=3049)),
+    ("er", dict(n=1500000, avg_degree=4.0, seed=3050)),
+    ("rmat", dict(scale=12, edge_factor=32, seed=3051)),
+    ("rmat", dict(scale=13, edge_factor=24, seed=3052, permute=True)),
+    ("rmat", dict(scale=15, edge_factor=8, seed=3053)),
+    ("rmat", dict(scale=16, edge_factor=32, seed=3054)),
+    ("rmat", dict(scale=14, edge_factor=8, seed=3055, directed=True)),
+    ("rmat", dict(scale=16, edge_factor=8, seed=3056, directed=True)),
+    ("rmat", dict(scale=18, edge_factor=24, seed=3057, directed=True)),
+    ("rmat", dict(scale=21, edge_factor=8, seed=3058)),
+    ("grid", dict(rows=40, cols=37, drop=0.1, seed=3059)),
+    ("er", dict(n=2097152, avg_degree=16.0, seed=3060)),
+    ("er", dict(n=1048576, avg_degree=16.0, seed=3061)),
+    ("er", dict(n=1048576, avg_degree=32.0, seed=3062)),
+    ("er", dict(n=524288, avg_degree=16.0, seed=3063)),
+    ("er", dict(n=262144, avg_degree=8.0, seed=3064)),
+    ("er", dict(n=262144, avg_degree=16.0, seed=3065)),
+    ("er", dict(n=3000000, avg_degree=8.0, seed=3066)),
+    ("er", dict(n=4194304, avg_degree=4.0, seed=3067)),
+    ("er", dict(n=4194304, avg_degree=8.0, seed=3068)),
+    ("er", dict(n=131072, avg_degree=16.0, seed=3069)),
+    ("er", dict(n=65536, avg_degree=8.0, seed=3070)),
+    ("er", dict(n=32768, avg_degree=16.0, seed=3071)),
+    ("er", dict(n=8192, avg_degree=24.0, seed=3072)),
+    ("er", dict(n=900000, avg_degree=4.0, seed=3073)),
+    ("er", dict(n=1048576, avg_degree=24.0, seed=3074)),
+    ("rmat", dict(scale=20, edge_factor=16, seed=3075)),
+    ("rmat", dict(scale=18, edge_factor=16, seed=3076)),
+    ("rmat", dict(scale=17, edge_factor=8, seed=3077)),
+    ("rmat", dict(scale=16, edge_factor=16, seed=3078, permute=True)),
+    ("rmat", dict(scale=19, edge_factor=24, seed=3079)),
+    ("rmat", dict(scale=21, edge_factor=16, seed=3080)),
+    ("rmat", dict(scale=12, edge_factor=8, seed=3081)),
+    ("rmat", dict(scale=20, edge_factor=8, seed=3082, directed=True)),
+    ("rmat", dict(scale=18, edge_factor=8, seed=3083, directed=True)),
+    ("rmat", dict(scale=15, edge_factor=16, seed=3084, directed=True)),
+    ("rmat", dict(scale=12, edge_factor=16, seed=3085, directed=True)),
+    ("rmat", dict(scale=20, edge_factor=24, seed=3086, directed=True)),
+    ("rmat", dict(scale=16, edge_factor=4, seed=3087)),
 ]
 
 
@@ -157,7 +218,25 @@ def load(csv_path: str):
     level = np.array([int(r["level"]) for r in rows])
     X = np.array([[int(r[f]) for f in FEATURES] for r in rows], dtype=np.int64).reshape(-1, NUM_FEATURES)
     T = np.array([[float(r[f"ms_{v}"]) for v in VARIANTS] for r in rows]).reshape(-1, NUM_VARIANTS)
-    return graph, root, level, X, T
+    return graph, root, level, X, leader_times(X, T)
+
+
+# On graphs whose out-degrees are at most LEADER_DEGREE the drivers expand a
+# level of at most LEADER_EDGES frontier edges on one cluster whichever push
+# the tree picks (bfs_small.cuh: 16 blocks x 1088 edges); the timing harness
+# times the whole-grid kernels. leader_times takes the cluster's time from the
+# 4096^2 grid (1.9 us below 2,000 frontier edges, 3.6 us at 15,900).
+LEADER_DEGREE, LEADER_EDGES = 8, 16 * 1088
+
+
+def leader_times(X, T):
+    """The times with every push variant's replaced by the cluster's where it runs."""
+    e = X[:, FEATURES.index("frontier_edges")]
+    small = (X[:, FEATURES.index("deg_max")] <= LEADER_DEGREE) & (e <= LEADER_EDGES)
+    push = [i for i, v in enumerate(VARIANTS) if v != "pull"]
+    T = T.copy()
+    T[np.ix_(small, push)] = (1.8e-3 + 0.115e-6 * e[small])[:, None]
+    return T
 
 
 def split_by_graph(graph, test_frac=0.3, seed=0):
@@ -174,17 +253,28 @@ def level_weights(T, trav, weighting):
     a level weighs its spread of times (slowest minus fastest), so splits go
     where a wrong choice costs most. 'relregret': that spread divided by the
     traversal's per-level-optimal time, the level's share of the traversal
-    slowdown that Table 2 averages."""
+    slowdown that Table 2 averages. 'cost': as 'relregret', with the spread cut
+    at four times the level's best (one whole-graph pull of a hub's list costs a
+    thousand levels) and half the step to the second best added, so that close
+    calls count too; its leaves are labelled by cost (fit)."""
     if weighting == "uniform":
         return np.ones(len(T))
     spread = T.max(axis=1) - T.min(axis=1) + 1e-5
     if weighting == "regret":
         return spread
-    opt = T.min(axis=1)
+    tot = traversal_optimum(T, trav)
+    if weighting == "cost":
+        s = np.sort(T, axis=1)
+        return (0.5 * (s[:, 1] - s[:, 0]) + np.minimum(s[:, -1] - s[:, 0], 4 * s[:, 0])) / tot + 1e-6
+    return spread / tot
+
+
+def traversal_optimum(T, trav):
+    """For every level, the per-level-optimal time of its whole traversal."""
     tot = {}
-    for k, t in zip(trav, opt):
+    for k, t in zip(trav, T.min(axis=1)):
         tot[k] = tot.get(k, 0.0) + t
-    return spread / np.array([tot[k] for k in trav])
+    return np.array([tot[k] for k in trav])
 
 
 # The library evaluates trees of up to 64 leaves in their bit-parallel form,
@@ -194,13 +284,20 @@ MAX_LEAVES = 64
 
 
 def fit(X, T, feature_idx, max_depth=8, min_samples_leaf=8, weighting="regret", trav=None, max_leaves=MAX_LEAVES):
-    """CART with Gini impurity (Section 2.1); labels: the fastest variant per level."""
+    """CART with Gini impurity (Section 2.1); labels: the fastest variant per level.
+    Under the 'cost' weighting each leaf is labelled with the variant of least
+    total time over its levels (each level's times over its traversal's optimum)
+    instead of the heaviest class: clf.leaf_label_, by node."""
     from sklearn.tree import DecisionTreeClassifier
     y = T.argmin(axis=1)
     w = level_weights(T, trav if trav is not None else np.zeros(len(T)), weighting)
     clf = DecisionTreeClassifier(criterion="gini", max_depth=max_depth, min_samples_leaf=min_samples_leaf,
                                  max_leaf_nodes=max_leaves, random_state=0)
     clf.fit(X[:, feature_idx], y, sample_weight=w)
+    if weighting == "cost":
+        cost = T / traversal_optimum(T, trav)[:, None]
+        leaf = clf.apply(X[:, feature_idx].astype(np.float32))
+        clf.leaf_label_ = {int(k): int(cost[leaf == k].sum(axis=0).argmin()) for k in np.unique(leaf)}
     return clf
 
 
@@ -215,7 +312,8 @@ def export(clf, feature_idx, path, meta=""):
             cls = clf.classes_
             top = int(cls[order[0]])
             tie = len(order) > 1 and math.isclose(float(v[order[0]]), float(v[order[1]]), rel_tol=1e-9)
-            lines.append(f"-1 0 -1 -1 {-1 if tie else top}")
+            labels = getattr(clf, "leaf_label_", None)
+            lines.append(f"-1 0 -1 -1 {labels[i] if labels else -1 if tie else top}")
         else:
             f = int(feature_idx[t.feature[i]])
             lines.append(f"{f} {int(math.floor(t.threshold[i]))} {t.children_left[i]} {t.children_right[i]} -1")
@@ -287,7 +385,7 @@ def evaluate(graph, root, level, X, T, nodes, mask=None):
 
 
 def cross_validate(graph, root, level, X, T, folds=6, depths=(6, 8, 10), feature_sets=None,
-                   weightings=("uniform", "regret", "relregret")):
+                   weightings=("uniform", "regret", "relregret", "cost")):
     """Mean held-out slowdown vs the per-level optimum, k folds split by graph."""
     import tempfile
     names = sorted(set(graph.tolist()))
@@ -406,19 +504,19 @@ def main():
     t.add_argument("--features", default="ext", choices=sorted(FEATURE_SETS))
     t.add_argument("--max-depth", type=int, default=8)
     t.add_argument("--min-leaf", type=int, default=8)
-    t.add_argument("--weighting", default="relregret", choices=["regret", "uniform", "relregret"])
+    t.add_argument("--weighting", default="relregret", choices=["regret", "uniform", "relregret", "cost"])
     t.add_argument("--all-graphs", action="store_true", help="train on every graph (no held-out split)")
     v = sub.add_parser("cv", help="k-fold cross-validation by graph over feature sets and weightings")
     v.add_argument("--csv", required=True)
     v.add_argument("--folds", type=int, default=6)
     v.add_argument("--features", nargs="*", default=None, choices=sorted(FEATURE_SETS))
-    v.add_argument("--weightings", nargs="*", default=["uniform", "regret", "relregret"])
+    v.add_argument("--weightings", nargs="*", default=["uniform", "regret", "relregret", "cost"])
     ls = sub.add_parser("level-split", help="the paper's random 70/30 split over levels: held-out accuracy")
     ls.add_argument("--csv", required=True)
     h = sub.add_parser("holdout", help="leave each graph family out in turn (Section 4.4 generality)")
     h.add_argument("--csv", required=True)
     h.add_argument("--features", default="ext_io", choices=sorted(FEATURE_SETS))
-    h.add_argument("--weighting", default="relregret", choices=["regret", "uniform", "relregret"])
+    h.add_argument("--weighting", default="relregret", choices=["regret", "uniform", "relregret", "cost"])
     h.add_argument("--max-depth", type=int, default=8)
     e = sub.add_parser("evaluate")
     e.add_argument("--csv", required=True)
