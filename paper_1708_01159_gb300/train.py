@@ -160,6 +160,34 @@ TRAIN_GRAPHS = [
     ("rmat", dict(scale=12, edge_factor=16, seed=3085, directed=True)),
     ("rmat", dict(scale=20, edge_factor=24, seed=3086, directed=True)),
     ("rmat", dict(scale=16, edge_factor=4, seed=3087)),
+    ("rmat", dict(scale=11, edge_factor=8, seed=3088)),
+    ("rmat", dict(scale=11, edge_factor=8, seed=3089, permute=True)),
+    ("rmat", dict(scale=11, edge_factor=16, seed=3090)),
+    ("rmat", dict(scale=11, edge_factor=16, seed=3091, permute=True)),
+    ("rmat", dict(scale=12, edge_factor=4, seed=3092)),
+    ("rmat", dict(scale=12, edge_factor=4, seed=3093, permute=True)),
+    ("rmat", dict(scale=12, edge_factor=4, seed=3094)),
+    ("rmat", dict(scale=12, edge_factor=4, seed=3095, permute=True)),
+    ("rmat", dict(scale=12, edge_factor=8, seed=3096)),
+    ("rmat", dict(scale=12, edge_factor=8, seed=3097, permute=True)),
+    ("rmat", dict(scale=12, edge_factor=16, seed=3098)),
+    ("rmat", dict(scale=12, edge_factor=16, seed=3099, permute=True)),
+    ("rmat", dict(scale=13, edge_factor=4, seed=3100)),
+    ("rmat", dict(scale=13, edge_factor=4, seed=3101, permute=True)),
+    ("rmat", dict(scale=13, edge_factor=4, seed=3102)),
+    ("rmat", dict(scale=13, edge_factor=4, seed=3103, permute=True)),
+    ("rmat", dict(scale=13, edge_factor=8, seed=3104)),
+    ("rmat", dict(scale=13, edge_factor=8, seed=3105, permute=True)),
+    ("rmat", dict(scale=13, edge_factor=16, seed=3106)),
+    ("rmat", dict(scale=13, edge_factor=16, seed=3107, permute=True)),
+    ("rmat", dict(scale=14, edge_factor=4, seed=3108)),
+    ("rmat", dict(scale=14, edge_factor=4, seed=3109, permute=True)),
+    ("rmat", dict(scale=14, edge_factor=8, seed=3110)),
+    ("rmat", dict(scale=14, edge_factor=8, seed=3111, permute=True)),
+    ("rmat", dict(scale=12, edge_factor=24, seed=3112)),
+    ("rmat", dict(scale=12, edge_factor=24, seed=3113, permute=True)),
+    ("rmat", dict(scale=11, edge_factor=32, seed=3114)),
+    ("rmat", dict(scale=11, edge_factor=32, seed=3115, permute=True)),
 ]
 
 
