@@ -450,12 +450,15 @@ __device__ __forceinline__ void stage_put_won(const Stage& s, int32_t* out, Tail
 }
 
 // Copies the staged entries out once at least `threshold` are waiting. Every
-// thread of the block must call it (it synchronises).
+// thread of the block must call it (it synchronises). Whether it copies is
+// decided in the barrier, from counts read before it: a thread that read the
+// count after the barrier could see what a faster one, already back from here,
+// had put for its next step, and copy alone. The thread that put last counts
+// its own entry, so the full count is among those read.
 template <typename TailT>
 __device__ __forceinline__ void stage_drain(const Stage& s, int32_t* out, TailT* tail, unsigned int threshold) {
-  __syncthreads();
+  if (!__syncthreads_or(min(*s.cnt, (unsigned)kStageCap) >= max(threshold, 1u))) return;
   const unsigned int c = min(*s.cnt, (unsigned)kStageCap);
-  if (c == 0 || c < threshold) return;  // uniform: every thread read the same count
   if (threadIdx.x == 0) *s.base = (unsigned int)atomicAdd(tail, (TailT)c);
   __syncthreads();
   const unsigned int b = *s.base;
