@@ -1026,7 +1026,9 @@ __device__ __forceinline__ void for_each_entry(const int32_t* off, int32_t n, in
       for (int32_t r = threadIdx.x; r < rows; r += blockDim.x) s_off[r] = off[r0 + r];
     __syncthreads();
     const int32_t* start = shared ? s_off : off + r0;
-    for (int32_t e = (int32_t)c0 + (int32_t)threadIdx.x; e < c1; e += blockDim.x) {
+    const int32_t len = c1 - (int32_t)c0;  // stepped from 0: an entry number past the end might not fit 32 bits
+    for (int32_t i = (int32_t)threadIdx.x; i < len; i += kThreads) {
+      const int32_t e = (int32_t)c0 + i;
       int32_t lo = 0, hi = rows - 1;
       while (lo < hi) {
         const int32_t mid = lo + (hi - lo + 1) / 2;
