@@ -280,7 +280,8 @@ __device__ void body_push_thread(const DevGraph& g, const Level& lv, const Stage
 // ---------------------------------------------------------------------------
 // Push, virtual warp of W lanes per frontier vertex (Section 3.1.3, after Hong
 // et al. 2011). Lanes stride the adjacency; W = 32 reads long lists with
-// 16-byte vector loads.
+// 16-byte vector loads. Positions in the lists that a step may carry past the
+// lists' end are unsigned: the end may lie 65 below 2^31.
 // ---------------------------------------------------------------------------
 template <int W>
 __device__ __forceinline__ void push_vwarp(const DevGraph& g, const Level& lv, const Stage& stage,
@@ -297,15 +298,15 @@ __device__ __forceinline__ void push_vwarp(const DevGraph& g, const Level& lv, c
     constexpr int kR = 4;
     const int grp = (int)threadIdx.x / W;
     for (int base = blockIdx.x * G * kR; base < lv.frontier; base += gridDim.x * G * kR) {
-      int32_t e[kR], end[kR];
+      uint32_t e[kR], end[kR];
 #pragma unroll
       for (int j = 0; j < kR; ++j) {
         const int i = base + grp * kR + j;
         e[j] = end[j] = 0;
         if (i < lv.frontier) {
           const int32_t u = lv.qin[i];
-          e[j] = g.off[u] + lane;
-          end[j] = g.off[u + 1];
+          e[j] = (uint32_t)(g.off[u] + lane);
+          end[j] = (uint32_t)g.off[u + 1];
         }
       }
       uint32_t valid;
@@ -336,7 +337,7 @@ __device__ __forceinline__ void push_vwarp(const DevGraph& g, const Level& lv, c
           int32_t v[1] = {beg + lane < a0 ? g.idx[beg + lane] : 0};
           visit_k<1>(g, lv, stage, v, beg + lane < a0 ? 1 : 0, edges);
         }
-        for (int32_t e = a0 + 4 * lane; e < a1; e += 128) {
+        for (uint32_t e = (uint32_t)(a0 + 4 * lane); e < (uint32_t)a1; e += 128) {
           const int4 q = *reinterpret_cast<const int4*>(g.idx + e);
           int32_t v[4] = {q.x, q.y, q.z, q.w};
           visit_k<4>(g, lv, stage, v, 4, edges);
@@ -346,14 +347,14 @@ __device__ __forceinline__ void push_vwarp(const DevGraph& g, const Level& lv, c
           visit_k<1>(g, lv, stage, v, a1 + lane < end ? 1 : 0, edges);
         }
       } else {
-        for (int32_t e = beg + lane; e < end; e += 4 * W) {
+        for (uint32_t e = (uint32_t)(beg + lane); e < (uint32_t)end; e += 4 * W) {
           int32_t v[4];
           int nv = 0;
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            const int32_t ek = e + k * W;
-            v[k] = ek < end ? g.idx[ek] : 0;
-            nv += ek < end ? 1 : 0;
+            const uint32_t ek = e + k * W;
+            v[k] = ek < (uint32_t)end ? g.idx[ek] : 0;
+            nv += ek < (uint32_t)end ? 1 : 0;
           }
           visit_k<4>(g, lv, stage, v, nv, edges);
         }
@@ -408,14 +409,14 @@ __device__ bool body_push_cta(const DevGraph& g, const Level& lv, const Stage& s
     if (end - beg < kCtaDirect) {
       // short lists: read directly; check the stage every 4th vertex (4 x 512
       // entries fit it), not after each one, to keep barriers rare
-      for (int32_t e = beg + tid; e < end; e += 4 * kThreads) {
+      for (uint32_t e = (uint32_t)beg + (uint32_t)tid; e < (uint32_t)end; e += 4 * kThreads) {  // unsigned as above
         int32_t v[4];
         int nv = 0;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          const int32_t ek = e + k * kThreads;
-          v[k] = ek < end ? g.idx[ek] : 0;
-          nv += ek < end ? 1 : 0;
+          const uint32_t ek = e + k * kThreads;
+          v[k] = ek < (uint32_t)end ? g.idx[ek] : 0;
+          nv += ek < (uint32_t)end ? 1 : 0;
         }
         visit_k<4>(g, lv, stage, v, nv, edges);
       }

@@ -29,13 +29,22 @@ def constant(path, name):
     return re.search(r"^(static )?constexpr [^\n]*\b" + name + r"\b = [^;]*;", text, re.M).group(0) + "\n"
 
 
-def run(tmp_path, source, *args, timeout=120):
-    """Compile `source` after host_cuda.h and run it: (exit status, output)."""
+def build(tmp_path, source):
+    """Compile `source` after host_cuda.h: the program's path."""
     src, exe = os.path.join(tmp_path, "t.cpp"), os.path.join(tmp_path, "t")
     with open(src, "w") as fh:
         fh.write('#include "host_cuda.h"\n' + source)
     r = subprocess.run(["g++", "-std=c++20", "-O1", "-w", "-fwrapv", "-pthread", "-I", HERE, src, "-o", exe],
                        capture_output=True, text=True)
     assert r.returncode == 0, r.stderr[-4000:]
+    return exe
+
+
+def execute(exe, *args, timeout=120):
+    """(exit status, output)"""
     r = subprocess.run([exe, *map(str, args)], capture_output=True, text=True, timeout=timeout)
     return r.returncode, r.stdout + r.stderr
+
+
+def run(tmp_path, source, *args):
+    return execute(build(tmp_path, source), *args)

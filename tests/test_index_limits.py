@@ -39,3 +39,84 @@ int main(int, char** argv) {
 def test_every_entry_of_the_last_chunk_once(tmp_path, m):
     rc, out = ds.run(str(tmp_path), CONSTANTS + ds.function("bfs_kernels.cu", "for_each_entry") + ENTRIES, m)
     assert rc == 0, (rc, out)
+
+
+# The push levels' own loops; the visits only count the edges they are given.
+PUSH_STUBS = r"""
+enum { CM_BLOCK, ST_TIMEOUT = 5 };
+struct Stage {};
+struct DevGraph { const int32_t *off, *idx; };
+struct Level { const int32_t* qin; int32_t frontier; };
+struct CtaPipe { int32_t* chunk; uint64_t* bar; uint32_t parity0, parity1, extra_tx; };
+inline void stage_flush(const Stage&, const Level&, unsigned int) {}
+inline void mbar_expect_tx(uint64_t*, uint32_t) {}
+inline void bulk_g2s(void*, const void*, uint32_t, uint64_t*) {}
+inline bool mbar_wait_bounded(uint64_t*, uint32_t) { return true; }
+volatile int32_t named;  // keeps the loads of the neighbours
+template <int K, int kCount = CM_BLOCK>
+void visit_km(const DevGraph&, const Level&, const Stage&, const int32_t (&v)[K], uint32_t valid, unsigned long long& e) {
+  for (int k = 0; k < K; ++k) named = v[k];
+  e += (unsigned)__builtin_popcount(valid);
+}
+template <int K, int kCount = CM_BLOCK>
+void visit_k(const DevGraph&, const Level&, const Stage&, const int32_t (&v)[K], int nv, unsigned long long& e) {
+  for (int k = 0; k < K; ++k) named = v[k];
+  e += (unsigned)max(nv, 0);
+}
+"""
+
+PUSH_BODIES = r"""
+// Edges the block visits, its threads one after another (no list long enough to be staged).
+static unsigned long long visited(int body, const DevGraph& g, const Level& lv) {
+  const Stage s{};
+  unsigned long long edges = 0;
+  blockDim.x = kThreads;
+  for (threadIdx.x = 0; threadIdx.x < kThreads; ++threadIdx.x) {
+    int32_t status = 0;
+    CtaPipe pp{};
+    switch (body) {
+      case 0: body_push_thread(g, lv, s, edges); break;
+      case 4: push_vwarp<4>(g, lv, s, edges); break;
+      case 8: push_vwarp<8>(g, lv, s, edges); break;
+      case 16: push_vwarp<16>(g, lv, s, edges); break;
+      case 32: push_vwarp<32>(g, lv, s, edges); break;
+      default: body_push_cta(g, lv, s, pp, &status, edges); break;
+    }
+  }
+  return edges;
+}
+"""
+
+LAST_ROW = r"""
+int main(int, char** argv) {
+  const int body = atoi(argv[1]);
+  const int32_t m = atoi(argv[2]), d = atoi(argv[3]);
+  const int32_t off[4] = {0, 400, m - d, m};  // vertex 0: 400 edges, vertex 2: the last d
+  const DevGraph g{off, guarded_zeros((int64_t)m + 8)};
+  const int32_t one[1] = {2};
+  if (visited(body, g, Level{one, 1}) != (unsigned)d) return 1;
+  // more vertices than the block has groups, long and short lists side by side
+  int32_t q[100];
+  for (int i = 0; i < 100; ++i) q[i] = i % 2 * 2;
+  return visited(body, g, Level{q, 100}) != 50ull * (400u + (unsigned)d);
+}
+"""
+
+PUSHES = [0, 4, 8, 16, 32, 99]  # thread, virtual warps, CTA
+
+
+def push_source():
+    names = ["body_push_thread", "push_vwarp", "body_push_cta"]
+    consts = [ds.constant("bfs_kernels.cu", "kLongList"), ds.constant("bfs_internal.cuh", "kStageCap")] + \
+        [ds.constant("bfs_kernels.cuh", k) for k in ("kCtaChunk", "kCtaDirect")]
+    return CONSTANTS + "".join(consts) + PUSH_STUBS + "".join(ds.function("bfs_kernels.cu", n) for n in names) + \
+        PUSH_BODIES
+
+
+@pytest.mark.parametrize("body", PUSHES)
+def test_pushes_visit_every_edge_of_the_last_row_once(tmp_path, body):
+    exe = ds.build(str(tmp_path), push_source() + LAST_ROW)
+    for m, d in [(5000, 7), (M_MAX, 1), (M_MAX, 5), (M_MAX - 3, 33), (M_MAX, 100), (M_MAX, 255), (M_MAX - 1, 300),
+                 (M_MAX, 511)]:
+        rc, out = ds.execute(exe, body, m, d)
+        assert rc == 0, (m, d, rc, out)
