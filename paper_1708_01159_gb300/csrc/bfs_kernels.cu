@@ -236,7 +236,9 @@ __device__ __forceinline__ int32_t warp_width(long long f, long long e, int32_t 
 // ---------------------------------------------------------------------------
 // Push, one thread per frontier vertex (Section 3.1.2 vertex push, over an
 // explicit queue instead of a scan of all vertices). Each thread walks its
-// vertex's adjacency four edges at a time.
+// vertex's adjacency four edges at a time. (Positions in a queue are unsigned
+// in all push variants: a frontier may have 2^31 - 3 vertices, and the step past
+// its end does not fit 31 bits then.)
 // ---------------------------------------------------------------------------
 // Lists from this length on are visited eight edges at a time, so that a hub's
 // thread has eight claims in flight (R-MAT 14 by vertex push alone, four roots:
@@ -245,10 +247,10 @@ constexpr int32_t kLongList = 32;
 
 template <int kCount = CM_BLOCK>
 __device__ void body_push_thread(const DevGraph& g, const Level& lv, const Stage& stage, unsigned long long& edges) {
-  const int stride = gridDim.x * blockDim.x;
-  for (int base = blockIdx.x * blockDim.x; base < lv.frontier; base += stride) {
-    const int i = base + threadIdx.x;
-    if (i < lv.frontier) {
+  const uint32_t stride = gridDim.x * blockDim.x, f = (uint32_t)lv.frontier;
+  for (uint32_t base = blockIdx.x * blockDim.x; base < f; base += stride) {
+    const uint32_t i = base + threadIdx.x;
+    if (i < f) {
       const int32_t u = lv.qin[i];
       const int32_t end = g.off[u + 1];
       int32_t e = g.off[u];
@@ -288,7 +290,8 @@ __device__ __forceinline__ void push_vwarp(const DevGraph& g, const Level& lv, c
                                            unsigned long long& edges) {
   constexpr int G = kThreads / W;  // groups per block
   const int lane = threadIdx.x & (W - 1);
-  if (W < 32 && lv.frontier > (int)gridDim.x * G) {
+  const uint32_t f = (uint32_t)lv.frontier;
+  if (W < 32 && f > gridDim.x * G) {
     // More frontier vertices than groups: a group takes kR consecutive
     // frontier vertices per step, and each round every lane visits one edge of
     // each of them (edge lane, lane + W, ...), so kR independent chains of
@@ -296,14 +299,14 @@ __device__ __forceinline__ void push_vwarp(const DevGraph& g, const Level& lv, c
     // (a high-diameter graph's levels on a narrow grid). A frontier that fits
     // one step keeps one vertex per group, spread over every block.
     constexpr int kR = 4;
-    const int grp = (int)threadIdx.x / W;
-    for (int base = blockIdx.x * G * kR; base < lv.frontier; base += gridDim.x * G * kR) {
+    const uint32_t grp = threadIdx.x / W;
+    for (uint32_t base = blockIdx.x * G * kR; base < f; base += gridDim.x * G * kR) {
       uint32_t e[kR], end[kR];
 #pragma unroll
       for (int j = 0; j < kR; ++j) {
-        const int i = base + grp * kR + j;
+        const uint32_t i = base + grp * kR + j;
         e[j] = end[j] = 0;
-        if (i < lv.frontier) {
+        if (i < f) {
           const int32_t u = lv.qin[i];
           e[j] = (uint32_t)(g.off[u] + lane);
           end[j] = (uint32_t)g.off[u + 1];
@@ -326,9 +329,9 @@ __device__ __forceinline__ void push_vwarp(const DevGraph& g, const Level& lv, c
     }
     return;
   }
-  for (int base = blockIdx.x * G; base < lv.frontier; base += gridDim.x * G) {
-    const int i = base + (int)threadIdx.x / W;
-    if (i < lv.frontier) {
+  for (uint32_t base = blockIdx.x * G; base < f; base += gridDim.x * G) {
+    const uint32_t i = base + threadIdx.x / W;
+    if (i < f) {
       const int32_t u = lv.qin[i];
       const int32_t beg = g.off[u], end = g.off[u + 1];
       if (W == 32 && end - beg >= 256) {
@@ -403,7 +406,7 @@ __device__ bool body_push_cta(const DevGraph& g, const Level& lv, const Stage& s
   const int tid = threadIdx.x;
   constexpr int kPer = kCtaChunk / kThreads;  // staged entries per thread per chunk
   int iter = 0;
-  for (int i = blockIdx.x; i < lv.frontier; i += gridDim.x, ++iter) {
+  for (uint32_t i = blockIdx.x; i < (uint32_t)lv.frontier; i += gridDim.x, ++iter) {
     const int32_t u = lv.qin[i];
     const int32_t beg = g.off[u], end = g.off[u + 1];
     if (end - beg < kCtaDirect) {
@@ -1074,8 +1077,8 @@ __global__ void k_undo_level(Buffers b, RunState* st) {
   const int32_t* qout = st->qsel ? b.q[0] : b.q[1];
   uint32_t* vis = st->vsel ? b.vis[1] : b.vis[0];
   int32_t* depth = st->depth;
-  const int stride = gridDim.x * blockDim.x;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < (int)count; i += stride) {
+  const uint32_t stride = gridDim.x * blockDim.x;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += stride) {
     const int32_t v = qout[i];
     depth[v] = -1;
     atomicAnd(&vis[v >> 5], ~(1u << (v & 31)));
@@ -1452,8 +1455,8 @@ __global__ void k_profile_reset(RunState* st, int32_t slot) {
 __global__ void k_undo_level_p(Buffers b, int32_t* depth, uint32_t qout, unsigned int count, uint32_t vsel) {
   const int32_t* q = qout ? b.q[1] : b.q[0];
   uint32_t* vis = vsel ? b.vis[1] : b.vis[0];
-  const int stride = gridDim.x * blockDim.x;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < (int)count; i += stride) {
+  const uint32_t stride = gridDim.x * blockDim.x;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += stride) {
     const int32_t v = q[i];
     depth[v] = -1;
     atomicAnd(&vis[v >> 5], ~(1u << (v & 31)));

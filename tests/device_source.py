@@ -12,7 +12,7 @@ CSRC = os.path.join(os.path.dirname(HERE), "paper_1708_01159_gb300", "csrc")
 def function(path, name):
     """The source text of function (or struct) `name`, its template line included."""
     text = open(os.path.join(CSRC, path)).read()
-    at = re.search(r"^(template <[^\n]*>\n)?(struct " + name + r" \{|[\w:<> \n_*&]*\b" + name + r"\()", text, re.M)
+    at = re.search(r"^(template <[^\n]*>\n)?(struct " + name + r" \{|\w[^\n;{}]*\b" + name + r"\()", text, re.M)
     assert at, f"{name} not found in {path}"
     pos = text.index("{", at.end() - 1)
     depth, end = 0, pos

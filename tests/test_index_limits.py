@@ -120,3 +120,58 @@ def test_pushes_visit_every_edge_of_the_last_row_once(tmp_path, body):
                  (M_MAX, 511)]:
         rc, out = ds.execute(exe, body, m, d)
         assert rc == 0, (m, d, rc, out)
+
+
+FULL_QUEUE = r"""
+int main(int, char** argv) {  // a frontier of f vertices without edges, the grid's last block
+  const int body = atoi(argv[1]);
+  const int32_t f = atoi(argv[2]);
+  const int32_t off[2] = {0, 0};
+  gridDim.x = 608;
+  blockIdx.x = 607;
+  return visited(body, DevGraph{off, nullptr}, Level{guarded_zeros(f), f}) != 0;
+}
+"""
+
+N_MAX = 2 ** 31 - 2  # bfs_graph_create's limit; a frontier has at most n - 1 vertices
+
+
+@pytest.mark.parametrize("body", PUSHES)
+def test_pushes_end_at_the_end_of_the_largest_queue(tmp_path, body):
+    exe = ds.build(str(tmp_path), push_source() + FULL_QUEUE)
+    for f in (1, 1000003, N_MAX - 1):
+        rc, out = ds.execute(exe, body, f)
+        assert rc == 0, (f, rc, out)
+
+
+UNDO = r"""
+struct Buffers { const int32_t* q[2]; uint32_t* vis[2]; };
+struct RunState { unsigned long long next_count; uint32_t qsel, vsel; int32_t* depth; };
+inline uint32_t atomicAnd(uint32_t* p, uint32_t x) { return __atomic_fetch_and(p, x, __ATOMIC_SEQ_CST); }
+"""
+
+UNDO_MAIN = r"""
+int main(int, char** argv) {
+  const unsigned int f = (unsigned)atoi(argv[1]);
+  const int32_t* q = guarded_zeros(f);
+  int32_t depth = 7;
+  uint32_t vis = ~0u;
+  RunState st{f, 0, 0, &depth};
+  const Buffers b{{q, q}, {&vis, &vis}};
+  gridDim.x = 1216;
+  blockIdx.x = 1215;
+  blockDim.x = kThreads;
+  for (threadIdx.x = 0; threadIdx.x < kThreads; ++threadIdx.x) {
+    k_undo_level(b, &st);
+    k_undo_level_p(b, &depth, 0, f, 0);
+  }
+  return 0;
+}
+"""
+
+
+def test_undo_ends_at_the_end_of_the_largest_queue(tmp_path):
+    src = CONSTANTS + UNDO + ds.function("bfs_kernels.cu", "k_undo_level") + \
+        ds.function("bfs_kernels.cu", "k_undo_level_p") + UNDO_MAIN
+    rc, out = ds.run(str(tmp_path), src, N_MAX - 1)
+    assert rc == 0, (rc, out)
