@@ -1618,7 +1618,7 @@ __global__ void k_tr_count(const int32_t* idx, int32_t m, int32_t* cnt) {
 // Generic exclusive scan of int32 (three kernels): per-block sums, scan of the
 // block sums, apply. Blocks of kThreads threads x kPeItems items.
 __global__ void __launch_bounds__(kThreads) k_scan_reduce(const int32_t* in, int32_t len, long long* bsum) {
-  const int nblk = (len + kPeTile - 1) / kPeTile;
+  const int nblk = (int)(((long long)len + kPeTile - 1) / kPeTile);  // len may lie 1 below 2^31 - 1
   for (int blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
     long long s = 0;
 #pragma unroll
@@ -1647,7 +1647,7 @@ __global__ void __launch_bounds__(kThreads) k_scan_top(long long* bsum, int32_t 
 
 __global__ void __launch_bounds__(kThreads) k_scan_apply(const int32_t* in, int32_t len, const long long* bsum,
                                                          int32_t* out) {
-  const int nblk = (len + kPeTile - 1) / kPeTile;
+  const int nblk = (int)(((long long)len + kPeTile - 1) / kPeTile);  // len may lie 1 below 2^31 - 1
   for (int blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
     const long long base = (long long)blk * kPeTile + threadIdx.x * kPeItems;
     int32_t d[kPeItems];

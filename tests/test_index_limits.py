@@ -175,3 +175,41 @@ def test_undo_ends_at_the_end_of_the_largest_queue(tmp_path):
         ds.function("bfs_kernels.cu", "k_undo_level_p") + UNDO_MAIN
     rc, out = ds.run(str(tmp_path), src, N_MAX - 1)
     assert rc == 0, (rc, out)
+
+
+SCAN = r"""
+template <typename T>
+T block_exclusive_scan(T x, T* total) {
+  *total = x;
+  return 0;
+}
+"""
+
+SCAN_MAIN = r"""
+int main(int, char** argv) {  // the block of the last entries alone
+  const int32_t len = atoi(argv[1]);
+  const int64_t nblk = ((int64_t)len + kPeTile - 1) / kPeTile;
+  std::vector<long long> bsum((size_t)nblk + 1, -1);
+  gridDim.x = 608;
+  blockIdx.x = (unsigned)((nblk - 1) % 608);
+  blockDim.x = kThreads;
+  const int32_t* in = guarded_zeros(len);
+  int32_t* out = (int32_t*)mmap(nullptr, ((size_t)len + 1) * 4, PROT_READ | PROT_WRITE,
+                                MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
+  if (out == MAP_FAILED) return 4;
+  threadIdx.x = 0;
+  k_scan_reduce(in, len, bsum.data());
+  if (bsum[(size_t)nblk - 1] != 0) return 1;  // its sum was written
+  bsum[(size_t)nblk] = 12345;
+  k_scan_apply(in, len, bsum.data(), out);
+  return out[len] != 12345;  // and the total
+}
+"""
+
+
+@pytest.mark.parametrize("n", [1, 2048, 2049, 2 ** 31 - 2047, N_MAX])
+def test_scan_reaches_its_last_block(tmp_path, n):
+    src = CONSTANTS + SCAN + ds.function("bfs_kernels.cu", "k_scan_reduce") + \
+        ds.function("bfs_kernels.cu", "k_scan_apply") + SCAN_MAIN
+    rc, out = ds.run(str(tmp_path), src, n)
+    assert rc == 0, (rc, out)
