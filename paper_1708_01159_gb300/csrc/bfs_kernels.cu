@@ -1290,7 +1290,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_bfs_persistent(const __grid_con
       break;
     }
     const int32_t v = forced >= 0 ? forced : tc.choose(g, L, f, (long long)e, discovered + f, prev);
-    if (kRecord > 0 && small_on && !force_full && v != V_PULL && small_fits(e, cluster_size())) {
+    if (kRecord > 0 && small_on && !force_full && v != V_PULL && small_fits(f, e, cluster_size())) {
       if (blockIdx.x < cluster_size()) {
         if (threadIdx.x == 0) {
           s_small.out.discovered = discovered;
@@ -1369,7 +1369,7 @@ __global__ void __launch_bounds__(kThreads) k_small_levels(const __grid_constant
   const long long discovered = st->discovered;
   // k_decide switches to the bitmap a pull level wrote; this kernel runs first
   const uint32_t vsel = st->vsel ^ (uint32_t)(st->level >= 0 && st->variant == V_PULL);
-  if (st->forced >= 0 || st->status != ST_OK || f == 0 || !small_fits(e, cluster_size())) return;  // uniform
+  if (st->forced >= 0 || st->status != ST_OK || f == 0 || !small_fits(f, e, cluster_size())) return;  // uniform
   const TreeChoice tc{st->tree_qs, st->tree, st->tree_nodes, 0, -1};
   const int32_t v = tc.choose(g, L, f, (long long)e, discovered + f, st->variant);
   if (v == V_PULL) return;  // uniform over the cluster: every block reads the same state

@@ -97,8 +97,12 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t pa
   return ok != 0u;
 }
 
-// Whether a level of e frontier edges is left to a leader of c blocks.
-__device__ __forceinline__ bool small_fits(unsigned long long e, uint32_t c) { return e <= c * kSmallEdges; }
+// Whether a level of f vertices and e frontier edges is left to a leader of c
+// blocks. The vertices count too: they are dealt out evenly when a run starts,
+// and a frontier of a directed graph may be a million vertices without an edge.
+__device__ __forceinline__ bool small_fits(unsigned int f, unsigned long long e, uint32_t c) {
+  return f <= c * (unsigned)kWonCap && e <= c * kSmallEdges;
+}
 
 // Vertex v's record: its W out-neighbours, -1 past its degree.
 template <int W>
@@ -255,7 +259,10 @@ __device__ __forceinline__ bool small_exchange(SmallShared& ss, uint32_t c, uint
   *leave = __any_sync(kFull, (unsigned)(m >> 48) & 1u) != 0;
   return __syncthreads_and(ok) != 0;
 }
-static_assert(kCandCap * 8 < (1 << 16) && kMaxCluster * kCandCap < (1 << 15), "message fields and their sums");
+// (a run's first exchange: kWonCap vertices a block at most, small_fits)
+static_assert(kCandCap * 8 < (1 << 16) && kMaxCluster * kCandCap < (1 << 15) && kWonCap * 8 < (1 << 16) &&
+                  kMaxCluster * kWonCap < (1 << 15),
+              "message fields and their sums");
 
 // Deal the candidates out again, candidate i of the whole cluster to block i %
 // c: a wavefront that started in one block spreads over the others. xc - 1 is
@@ -371,7 +378,7 @@ __device__ __noinline__ void small_run(const DevGraph& g, const Buffers& b, uint
     if (!ok || leave || f == 0u) break;
     if (t.L > n || t.discovered > n) break;  // corrupted state: the caller reports it
     v = tc.choose(g, t.L, f, (long long)e, t.discovered + f, t.prev);
-    if (v == V_PULL || !small_fits(e, c)) break;
+    if (v == V_PULL || !small_fits(f, e, c)) break;
     t.discovered += f;
     t.reached += (long long)e;
     // dealt out when one block has twice its share, or needs a step more than they do
