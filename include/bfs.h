@@ -350,10 +350,11 @@ int bfs_batch_tune_ex(bfs_graph_t g, const int32_t* roots, int32_t k, int32_t* d
  * the one array, which keeps the previous call's contents (each call clears
  * what it reads first): calls whose work overlaps on the GPU, from any stream
  * or thread, race and corrupt each other, so serialise them. The CSR is
- * validated on every call (BFS_ERR_BAD_GRAPH). Synchronous: one cooperative
- * launch validates and traverses, then its status is read back. Every level is
- * the edge-centric push (no tree switching). BFS_ERR_TIMEOUT if a bounded
- * device-side wait gave up.
+ * validated on every call (BFS_ERR_BAD_GRAPH). Synchronous: ordinary launches
+ * (none cooperative, so the call runs beside other kernels on whatever part of
+ * the GPU they leave free), the status read back after the first 8 to 20 levels
+ * and then each time half as many again have run. Every level is the
+ * edge-centric push (no tree switching).
  */
 int bfs_run_static(const int32_t* row_offsets, const int32_t* col_indices, int64_t n, int64_t m, int32_t root,
                    int32_t* depth_out, bfs_stream_t stream);
