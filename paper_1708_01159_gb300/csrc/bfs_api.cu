@@ -195,6 +195,7 @@ struct Shapes {
   int init, push_thread, push_warp, push_cta, push_edge, pull, edge_list;
   int cluster;  // blocks per cluster of the persistent kernel (1: none)
   int persist;  // cooperative grid of the persistent kernel (0: not supported)
+  int forced;   // the same of a forced variant's run, which has no small levels and no clusters
   int profile;  // cooperative grid of the per-level timing kernel (the persistent grid when it fits)
 };
 
@@ -747,8 +748,14 @@ int launch_persistent(bfs_graph* g, Workspace* ws, int32_t root, int32_t* depth,
   uint32_t epoch = ++ws->epoch;  // runs on one workspace are ordered, so consecutive launches differ
   int32_t stall = take_stall();
   void* args[] = {&dg, &b, &st, &depth, &root, &forced, &tree, &nodes, &qs, &epoch, &stall};
-  const int grid = grid_blocks > 0 ? std::min(grid_blocks, g->shapes.persist) : g->shapes.persist;
-  int cluster = g->shapes.cluster;
+  // A forced variant runs as itself at every level, so it needs no cluster, and
+  // takes the blocks that clusters leave out. 528 in clusters -> 608: pull forced
+  // on 2^24 vertices of out-degree 8 5.62 -> 4.92 ms, virtual warps 1.83 -> 1.69;
+  // where a level is only latency the larger barrier costs some of it back (777 x
+  // 1021 grid, virtual warps 8.28 -> 8.45 ms).
+  const int full = forced >= 0 ? g->shapes.forced : g->shapes.persist;
+  const int grid = grid_blocks > 0 ? std::min(grid_blocks, full) : full;
+  int cluster = forced >= 0 ? 1 : g->shapes.cluster;
   while (cluster > 1 && grid % cluster) cluster /= 2;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeCooperative;
@@ -762,7 +769,7 @@ int launch_persistent(bfs_graph* g, Workspace* ws, int32_t root, int32_t* depth,
   cfg.stream = stream;
   cfg.attrs = at;
   cfg.numAttrs = cluster > 1 ? 2 : 1;
-  CU(cudaLaunchKernelExC(&cfg, persistent_kernel(dg.rec_w), args));
+  CU(cudaLaunchKernelExC(&cfg, persistent_kernel(cluster > 1 ? dg.rec_w : 0), args));
   return BFS_OK;
 }
 
@@ -1383,12 +1390,12 @@ int bfs_graph_create(const int32_t* row_offsets, const int32_t* col_indices, int
   // the persistent kernel needs every block resident: one full occupancy wave
   int coop = 0, per_sm = 0;
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, g->device);
-  void* const persistent = persistent_kernel(dg.rec_w);
-  if (coop && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persistent, kThreads, 0) == cudaSuccess &&
+  if (coop && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persistent_kernel(0), kThreads, 0) == cudaSuccess &&
       per_sm > 0)
     s.persist = g->sms * std::min(per_sm, 8);
   else
     s.persist = 0;
+  s.forced = s.persist;
   // Graphs with vertex records run their small levels on one cluster, so their
   // grid is launched in clusters. Clusters of 16 blocks leave 80 of the 608
   // blocks of a GB300 out (8: 16 of them); a 4096^2 grid traversal takes 17 ms
@@ -1397,6 +1404,7 @@ int bfs_graph_create(const int32_t* row_offsets, const int32_t* col_indices, int
   s.cluster = 1;
   if (s.persist > 0 && dg.rec_w > 0) {
     const int want = kMaxCluster;
+    void* const persistent = persistent_kernel(dg.rec_w);
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)want;
@@ -1410,9 +1418,10 @@ int bfs_graph_create(const int32_t* row_offsets, const int32_t* col_indices, int
     if (cudaFuncSetAttribute(persistent, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
         cudaFuncSetAttribute(small_levels_kernel(dg.rec_w), cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
             cudaSuccess &&
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persistent, kThreads, 0) == cudaSuccess &&
         cudaOccupancyMaxActiveClusters(&clusters, persistent, &cfg) == cudaSuccess && clusters > 0) {
       s.cluster = want;
-      s.persist = std::min(s.persist / want, clusters) * want;
+      s.persist = std::min(g->sms * std::min(per_sm, 8) / want, clusters) * want;
     }
   }
   per_sm = 0;
