@@ -169,6 +169,13 @@ int parse_tree(const std::string& text, std::vector<TreeNode>* out) {
 // ---------------------------------------------------------------------------
 // Workspaces
 // ---------------------------------------------------------------------------
+// The level loop as a CUDA graph, and its conditional handles.
+struct LevelGraph {
+  cudaGraph_t graph = nullptr;
+  cudaGraphExec_t exec = nullptr;
+  unsigned long long h_while = 0, h_switch = 0;
+};
+
 struct Workspace {
   Buffers b{};
   RunState* st = nullptr;
@@ -178,9 +185,7 @@ struct Workspace {
   long long* log_time = nullptr;
   int32_t log_cap = 0;
   int32_t* host_depth_stage = nullptr;  // device buffer for runs whose output is host memory
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t exec = nullptr;
-  cudaGraphNode_t start_node = nullptr;
+  LevelGraph loop, loop_forced;  // of tree-driven runs and of forced variants' (built when first used)
   cudaEvent_t done = nullptr;
   cudaStream_t last_stream = nullptr;
   uint32_t epoch = 0;  // persistent launches so far (the kernel's barrier-state reset handshake)
@@ -289,8 +294,10 @@ int upload_now(const bfs_graph* g, void* dst, const void* src, size_t bytes) {
 
 void free_workspace(Workspace* ws) {
   if (!ws) return;
-  if (ws->exec) cudaGraphExecDestroy(ws->exec);
-  if (ws->graph) cudaGraphDestroy(ws->graph);
+  for (LevelGraph* lg : {&ws->loop, &ws->loop_forced}) {
+    if (lg->exec) cudaGraphExecDestroy(lg->exec);
+    if (lg->graph) cudaGraphDestroy(lg->graph);
+  }
   if (ws->done) cudaEventDestroy(ws->done);
   for (void* p : ws->allocs) cudaFree(p);
   delete ws;
@@ -325,13 +332,9 @@ int add_kernel(cudaGraph_t graph, cudaGraphNode_t* node, const cudaGraphNode_t* 
   return BFS_OK;
 }
 
-// The workspace's device state before its first run: the log buffers and, once
-// the level-loop graph exists, its conditional handles.
-int init_run_state(const bfs_graph* g, Workspace* ws, unsigned long long h_while, unsigned long long h_switch) {
+// The workspace's device state before its first run: the log buffers.
+int init_run_state(const bfs_graph* g, Workspace* ws) {
   RunState init{};
-  init.h_while = h_while;
-  init.h_switch = h_switch;
-  init.use_handles = h_while != 0;
   init.log_cap = ws->log_cap;
   init.log_variant = ws->log_variant;
   init.log_frontier = ws->log_frontier;
@@ -343,28 +346,31 @@ int init_run_state(const bfs_graph* g, Workspace* ws, unsigned long long h_while
 // Build the level loop of one workspace as a CUDA graph with conditional nodes
 // (on the workspace's first run in the graph driver).
 // The graph holds the level loop only: k_loop_start opens the WHILE loop on the
-// device, and per-run values (root, output, forced variant, tree) reach it
-// through RunState, written by a k_init launched on the same stream just
-// before. Nothing in the instantiated graph changes between launches, so
-// back-to-back launches on one stream cannot see each other's parameters.
-int build_graph(bfs_graph* g, Workspace* ws) {
-  CU(cudaGraphCreate(&ws->graph, 0));
+// device, and per-run values (root, output, forced variant, tree, the graph's
+// handles) reach it through RunState, written by a k_init launched on the same
+// stream just before. Nothing in the instantiated graph changes between launches,
+// so back-to-back launches on one stream cannot see each other's parameters.
+// has_small: with the kernel that runs small levels before each decision.
+int build_graph(const bfs_graph* g, Workspace* ws, bool has_small, LevelGraph* lg) {
+  if (lg->graph) cudaGraphDestroy(lg->graph);  // of an attempt that failed
+  lg->graph = nullptr;
+  CU(cudaGraphCreate(&lg->graph, 0));
   KArgs ka{g->dg, ws->b, ws->st, {}};
-  TRY(add_kernel(ws->graph, &ws->start_node, nullptr, reinterpret_cast<const void*>(&k_loop_start), 1, 32, ka));
+  cudaGraphNode_t start;
+  TRY(add_kernel(lg->graph, &start, nullptr, reinterpret_cast<const void*>(&k_loop_start), 1, 32, ka));
 
   cudaGraphConditionalHandle hw;
-  CU(cudaGraphConditionalHandleCreate(&hw, ws->graph, 0, 0));
+  CU(cudaGraphConditionalHandleCreate(&hw, lg->graph, 0, 0));
   cudaGraphNodeParams wp{};
   wp.type = cudaGraphNodeTypeConditional;
   wp.conditional.handle = hw;
   wp.conditional.type = cudaGraphCondTypeWhile;
   wp.conditional.size = 1;
   cudaGraphNode_t wnode;
-  CU(cudaGraphAddNode(&wnode, ws->graph, &ws->start_node, nullptr, 1, &wp));
+  CU(cudaGraphAddNode(&wnode, lg->graph, &start, nullptr, 1, &wp));
   cudaGraph_t body = wp.conditional.phGraph_out[0];
 
   cudaGraphNode_t decide, small;
-  const bool has_small = g->shapes.cluster > 1;
   if (has_small) {
     TRY(add_kernel(body, &small, nullptr, small_levels_kernel(g->dg.rec_w), g->shapes.cluster, kThreads, ka));
     cudaKernelNodeAttrValue cl{};
@@ -402,9 +408,10 @@ int build_graph(bfs_graph* g, Workspace* ws) {
                  ka));
   TRY(add_kernel(vb[V_REV_EDGE_LIST], &n0, nullptr, reinterpret_cast<const void*>(&k_rev_edge_list), s.edge_list,
                  kThreads, ka));
-  CU(cudaGraphInstantiate(&ws->exec, ws->graph, 0));
-  // the handles live in the device state, where decide sets them each level
-  return init_run_state(g, ws, hw, hs);
+  lg->h_while = hw;
+  lg->h_switch = hs;
+  CU(cudaGraphInstantiate(&lg->exec, lg->graph, 0));
+  return BFS_OK;
 }
 
 int create_workspace(bfs_graph* g, Workspace** out) {
@@ -435,7 +442,7 @@ int create_workspace(bfs_graph* g, Workspace** out) {
     cudaError_t e = cudaEventCreateWithFlags(&ws->done, cudaEventDisableTiming);
     if (e != cudaSuccess) r = fail(BFS_ERR_CUDA, "cudaEventCreate: %s", cudaGetErrorString(e));
   }
-  if (r == BFS_OK) r = init_run_state(g, ws, 0, 0);
+  if (r == BFS_OK) r = init_run_state(g, ws);
   if (r != BFS_OK) {
     free_workspace(ws);
     return r;
@@ -721,16 +728,15 @@ int ensure_origin(bfs_graph* g) {
 int launch_variant(bfs_graph* g, Workspace* ws, int v, cudaStream_t s, int32_t count_mode = CM_BLOCK);
 
 int launch_graph(bfs_graph* g, Workspace* ws, int32_t root, int32_t* depth, int32_t forced, cudaStream_t stream) {
-  if (!ws->exec) {
-    // first graph-driver run on this workspace: its previous runs (other
-    // drivers) finish before the state they use is rewritten
-    CU(cudaEventSynchronize(ws->done));
-    TRY(build_graph(g, ws));
-  }
+  // a forced variant has no small levels: its loop is a graph without their
+  // kernel (777 x 1021 grid, 1,515 levels of virtual warps: 26.2 ms with it, 24.1 without)
+  const bool small = g->shapes.cluster > 1;
+  LevelGraph* lg = small && forced >= 0 ? &ws->loop_forced : &ws->loop;
+  if (!lg->exec) TRY(build_graph(g, ws, small && forced < 0, lg));
   k_init<<<g->shapes.init, kThreads, 0, stream>>>(g->dg, ws->b, ws->st, depth, root, forced, g->tree, g->tree_nodes,
-                                                  g->tree_qs, 1);
+                                                  g->tree_qs, 1, lg->h_while, lg->h_switch);
   CU(cudaGetLastError());
-  CU(cudaGraphLaunch(ws->exec, stream));
+  CU(cudaGraphLaunch(lg->exec, stream));
   return BFS_OK;
 }
 
@@ -778,7 +784,7 @@ int launch_persistent(bfs_graph* g, Workspace* ws, int32_t root, int32_t* depth,
 int launch_host_loop(bfs_graph* g, Workspace* ws, int32_t root, int32_t* depth, int32_t forced, cudaStream_t s,
                      int32_t count_mode) {
   k_init<<<g->shapes.init, kThreads, 0, s>>>(g->dg, ws->b, ws->st, depth, root, forced, g->tree, g->tree_nodes,
-                                             g->tree_qs, 0);
+                                             g->tree_qs, 0, 0, 0);
   CU(cudaGetLastError());
   RunState hs{};
   for (;;) {
@@ -1076,7 +1082,7 @@ int profile_levels_persistent(bfs_graph* g, Workspace* ws, int32_t root, int32_t
     tree = ts.nodes;
   }
   k_init<<<g->shapes.init, kThreads, 0, s>>>(g->dg, ws->b, ws->st, depth, root, -1, g->tree, g->tree_nodes,
-                                             g->tree_qs, 0);
+                                             g->tree_qs, 0, 0, 0);
   CU(cudaGetLastError());
   int32_t host_root = root;
   int32_t ends[2] = {0, 0};
@@ -1807,7 +1813,7 @@ int bfs_profile_levels(bfs_graph_t g, int32_t root, int32_t reps, int32_t advanc
   std::vector<float> t(reps);
   auto body = [&]() -> int {
     k_init<<<g->shapes.init, kThreads, 0, s>>>(g->dg, ws->b, ws->st, depth, root, -1, g->tree, g->tree_nodes,
-                                               g->tree_qs, 0);
+                                               g->tree_qs, 0, 0, 0);
     CU(cudaGetLastError());
     RunState hs{};
     for (;;) {

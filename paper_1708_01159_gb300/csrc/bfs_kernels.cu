@@ -798,7 +798,8 @@ __device__ void body_edge_list(const DevGraph& g, const Level& lv, const Stage& 
 // ===========================================================================
 __global__ void __launch_bounds__(kThreads) k_init(DevGraph g, Buffers b, RunState* st, int32_t* depth, int32_t root,
                                                    int32_t forced, const TreeNode* tree, int32_t tree_nodes,
-                                                   const QsTree* tree_qs, int32_t use_handles) {
+                                                   const QsTree* tree_qs, int32_t use_handles,
+                                                   unsigned long long h_while, unsigned long long h_switch) {
   if (blockIdx.x == 0 && threadIdx.x == 0) st->t_entry = (long long)global_ns();
   init_fill(g, b.vis[0], depth, root);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -808,6 +809,8 @@ __global__ void __launch_bounds__(kThreads) k_init(DevGraph g, Buffers b, RunSta
     st->tree_nodes = tree_nodes;
     st->root = root;
     st->forced = forced;
+    st->h_while = h_while;
+    st->h_switch = h_switch;
     st->use_handles = use_handles;
     st->level = -1;
     st->variant = -1;

@@ -16,7 +16,8 @@ constexpr int kHeavy = 1024;        // degree from which an edge-centric level d
 constexpr int kHeavyCap = 1 << 16;  // most vertices an edge-centric level sets aside
 
 __global__ void k_init(DevGraph g, Buffers b, RunState* st, int32_t* depth, int32_t root, int32_t forced,
-                       const TreeNode* tree, int32_t tree_nodes, const QsTree* tree_qs, int32_t use_handles);
+                       const TreeNode* tree, int32_t tree_nodes, const QsTree* tree_qs, int32_t use_handles,
+                       unsigned long long h_while, unsigned long long h_switch);
 __global__ void k_decide(DevGraph g, Buffers b, RunState* st);
 __global__ void k_loop_start(DevGraph g, Buffers b, RunState* st);
 __global__ void k_push_thread(DevGraph g, Buffers b, RunState* st);
