@@ -308,6 +308,9 @@ __device__ __forceinline__ uint32_t ld_nc_u32(const uint32_t* p) {
 // predicated instruction each, so that several in a row are in flight
 // together: with an `if` around each, the compiler branches around them and
 // waits for one's result before it issues the next.
+// ld_if is for arrays that no launch writes (the graph's): to the compiler its
+// result follows from its operands alone, so it may move it over a barrier or take
+// one load's result for a later one's.
 __device__ __forceinline__ int32_t ld_if(bool p, const int32_t* a, int32_t otherwise) {
   int32_t x = otherwise;
   asm("{\n .reg .pred q;\n setp.ne.s32 q, %2, 0;\n @q ld.global.s32 %0, [%1];\n}\n"
@@ -316,7 +319,8 @@ __device__ __forceinline__ int32_t ld_if(bool p, const int32_t* a, int32_t other
   return x;
 }
 
-// The same, issued where it stands (the compiler moves the one above to its use).
+// The same, issued where it stands, for anything a launch writes (queues, lists,
+// bitmaps) too.
 __device__ __forceinline__ int32_t ld_now_if(bool p, const int32_t* a, int32_t otherwise) {
   int32_t x = otherwise;
   asm volatile("{\n .reg .pred q;\n setp.ne.s32 q, %2, 0;\n @q ld.global.s32 %0, [%1];\n}\n"

@@ -193,7 +193,7 @@ __device__ __forceinline__ int32_t pe_scan_all(const DevGraph& g, const int32_t*
 #pragma unroll
   for (int k = 0; k < kPeItems; ++k) {
     const int i = k * kThreads + (int)threadIdx.x;
-    const int32_t u = ld_if(i < f, q + (i < f ? i : 0), -1);
+    const int32_t u = ld_now_if(i < f, q + (i < f ? i : 0), -1);
     beg[k] = ld_if(u >= 0, g.off + (u >= 0 ? u : 0), 0);
     d[k] = ld_if(u >= 0, g.off + (u >= 0 ? u : 0) + 1, 0);
   }

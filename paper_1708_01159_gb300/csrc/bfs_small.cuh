@@ -326,7 +326,7 @@ __device__ __noinline__ void small_run(const DevGraph& g, const Buffers& b, uint
   for (unsigned int base = 0; base < t.f; base += c * kThreads) {
     const unsigned int i = base + rank + c * (unsigned)tid;
     const bool have[1] = {i < t.f};
-    const int32_t u[1] = {ld_if(have[0], qin + i, 0)};
+    const int32_t u[1] = {ld_now_if(have[0], qin + i, 0)};
     const int32_t none[1] = {-2};
     int32_t r[1][W];
     ld_record_if<W>(have[0], rec, u[0], r[0]);
