@@ -503,7 +503,12 @@ int bfs_debug_fail_alloc_after(int n);
  * launch's first grid barrier expects one arrival more than the grid has;
  * mode 2: the first level-ending barrier of a traversal, likewise; mode 3: the
  * first adjacency copy staged by the CTA push expects 16 bytes more than it
- * copies (a level the CTA push expands with a list of 512 entries or more).
+ * copies (a level the CTA push expands with a list of 512 entries or more);
+ * modes 5 and 6, on graphs whose out-degrees are at most 8, where a cluster of
+ * blocks expands the small levels: the second exchange of counts within the
+ * cluster expects one arrival too many in one block (5), or the other blocks are
+ * not told the state the first run of small levels ends in (6); a launch without
+ * such levels ends normally. There is no mode 4.
  * Every wait of the library is bounded (about 2 s), so the kernel gives up,
  * records BFS_ERR_TIMEOUT in its status word (bfs_run_ex with stats, or
  * bfs_run_batch with edges_out, returns it) and exits; the next launch on the

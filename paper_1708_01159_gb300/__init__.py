@@ -423,7 +423,8 @@ def bfs_profile_levels(g: int, root: int, reps: int = 5, advance_variant: int = 
 def bfs_debug_stall_next_launch(mode: int) -> None:
     """Test hook: the next persistent traversal or multi-source wave lets one
     bounded device wait run out (1 first grid barrier, 2 first level barrier,
-    3 first staged copy of the CTA push; 0 clears), so the run reports
+    3 first staged copy of the CTA push, 5 second count exchange and 6 published
+    state of the cluster that runs small levels; 0 clears), so the run reports
     BFS_ERR_TIMEOUT after about 2 s instead of finishing."""
     _check(lib().bfs_debug_stall_next_launch(int(mode)), "bfs_debug_stall_next_launch")
 

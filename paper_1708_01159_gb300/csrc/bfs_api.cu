@@ -1204,7 +1204,8 @@ int bfs_debug_fail_alloc_after(int n) {
 }
 
 int bfs_debug_stall_next_launch(int mode) {
-  if (mode < STALL_NONE || mode > STALL_BULK_COPY) return fail(BFS_ERR_INVALID_ARG, "stall mode %d", mode);
+  if (mode < STALL_NONE || (mode > STALL_BULK_COPY && mode < STALL_LEADER_MESSAGE) || mode > STALL_LEADER_STATE)
+    return fail(BFS_ERR_INVALID_ARG, "stall mode %d", mode);
   g_stall_next.store(mode);
   return BFS_OK;
 }

@@ -87,6 +87,9 @@ enum Stall : int32_t {
   STALL_GRID_BARRIER = 1,   // the first grid barrier expects one arrival more than the grid has
   STALL_LEVEL_BARRIER = 2,  // the first level-ending barrier of a traversal, likewise
   STALL_BULK_COPY = 3,      // the first staged adjacency copy of the CTA push expects 16 bytes more than it copies
+  // small levels (bfs_small.cuh); a launch that runs none ends normally
+  STALL_LEADER_MESSAGE = 5,  // the leader's last block expects one arrival too many on its second message exchange
+  STALL_LEADER_STATE = 6,    // the leader does not publish the state its first run of small levels ends in
 };
 
 // Section 4.1: an unknown prediction at the first level falls back to the

@@ -1256,8 +1256,12 @@ __global__ void __launch_bounds__(kThreads, 4) k_bfs_persistent(const __grid_con
   }
   if (threadIdx.x == 0) {
     s_log = RunLog{st->log_cap, st->log_variant, st->log_frontier, st->log_edges, st->log_time};
+    const bool late = kRecord > 0 && stall == STALL_LEADER_MESSAGE && blockIdx.x + 1u == cluster_size();
     mbar_init(&s_small.bar[0], 1);
-    mbar_init(&s_small.bar[1], 1);
+    mbar_init(&s_small.bar[1], late ? 2 : 1);
+    s_small.failed = s_small.run_no = 0u;
+    for (int i = 0; i < kMaxCluster; ++i) s_small.ended[i] = 0u;
+    s_small.mute = stall == STALL_LEADER_STATE ? 1u : 0u;
   }
   cta_pipe_init(bar);
   CtaPipe pp{ubuf, bar, 0u, 0u, stall == STALL_BULK_COPY ? 16u : 0u};
@@ -1268,9 +1272,9 @@ __global__ void __launch_bounds__(kThreads, 4) k_bfs_persistent(const __grid_con
       if (global_ns() - t0 > kWaitLimitNs) break;  // the first barrier then times out and reports it
   }
   // small levels go to cluster 0 when the tree drives the run (a forced
-  // variant is timed as itself; a stalled launch keeps its barriers)
-  const bool small_on =
-      kRecord > 0 && forced < 0 && stall == STALL_NONE && cluster_size() > 1u && cluster_size() <= (uint32_t)kMaxCluster;
+  // variant is timed as itself; a launch whose grid barriers are stalled keeps them)
+  const bool small_on = kRecord > 0 && forced < 0 && (stall == STALL_NONE || stall >= STALL_LEADER_MESSAGE) &&
+                        cluster_size() > 1u && cluster_size() <= (uint32_t)kMaxCluster;
   uint32_t vsel = 0;
   uint32_t slot = 0;  // level words: this level's slot (the levels run on the whole grid, modulo 3)
   const TreeChoice tc{use_qs ? &s_qs : nullptr, tree, tree_nodes, 0, -1};
@@ -1350,7 +1354,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_bfs_persistent(const __grid_con
     st->edges_reached = s_small.out.reached;
   }
   // no block of a cluster ends while another may still send to its shared memory
-  if (kRecord > 0 && cluster_size() > 1u) cluster_barrier();
+  if (kRecord > 0 && cluster_size() > 1u) small_end(s_small, cluster_size(), cluster_rank(), ~0u, ok);
 }
 
 // Graph driver, before each level's decision, for graphs with vertex records
@@ -1379,6 +1383,8 @@ __global__ void __launch_bounds__(kThreads) k_small_levels(const __grid_constant
   if (threadIdx.x == 0) {
     s_log = RunLog{st->log_cap, st->log_variant, st->log_frontier, st->log_edges, st->log_time};
     s_small.out = TravState{discovered, st->edges_reached, e, f, L, st->variant, 0, 1, 0u};
+    s_small.failed = s_small.mute = s_small.run_no = 0u;
+    for (int i = 0; i < kMaxCluster; ++i) s_small.ended[i] = 0u;
     mbar_init(&s_small.bar[0], 1);
     mbar_init(&s_small.bar[1], 1);
     mbar_fence_init();

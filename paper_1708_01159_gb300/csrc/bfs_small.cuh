@@ -56,6 +56,11 @@ struct SmallShared {
   unsigned int part_f[kThreads / 32], part_e[kThreads / 32];
   unsigned int runs;  // small runs so far (the blocks that wait count them)
   TravState out;
+  unsigned int run_no;              // leader: small runs so far
+  unsigned int ended[kMaxCluster];  // each block of the cluster: the last run it has ended, ~0 after its last level
+                                    // (written by that block)
+  unsigned int failed;              // a block of the cluster gave a wait up (written by that block)
+  unsigned int mute;                // test hook: the state is not published
 };
 
 __device__ __forceinline__ uint32_t cluster_size() {
@@ -77,6 +82,9 @@ __device__ __forceinline__ Candidate ld_cluster(uint32_t addr) {
   Candidate x;
   asm volatile("ld.shared::cluster.v2.s32 {%0, %1}, [%2];" : "=r"(x.v), "=r"(x.from) : "r"(addr) : "memory");
   return x;
+}
+__device__ __forceinline__ void st_cluster_u32(uint32_t addr, unsigned int x) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(x) : "memory");
 }
 __device__ __forceinline__ void st_async_u64(uint32_t addr, unsigned long long x, uint32_t bar) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(addr), "l"(x),
@@ -286,11 +294,33 @@ __device__ __forceinline__ void small_deal(SmallShared& ss, uint32_t c, uint32_t
   cluster_barrier();  // every block has read what it takes
 }
 
+// The end of small run `no`, for every block of the leader, and (~0) of the levels,
+// for every block of a cluster: true when none has given a wait up. A block that
+// did is here before the others, who may be dealing, or at the end of a run it did
+// not start: their barriers are answered until they have given up waiting for its
+// messages and have come here too. So no block leaves, let alone ends, while
+// another may still send to its shared memory. (Telling the others of the failure
+// in the dealing's barrier instead cost every level 0.5 to 1 %.)
+__device__ __forceinline__ bool small_end(SmallShared& ss, uint32_t c, uint32_t rank, unsigned int no, bool ok) {
+  if (threadIdx.x < c) {
+    if (!ok) st_cluster_u32(map_rank(smem_u32(&ss.failed), threadIdx.x), 1u);
+    st_cluster_u32(map_rank(smem_u32(&ss.ended[rank]), threadIdx.x), no);
+  }
+  __syncwarp();
+  bool here;  // the block of this lane is
+  do {
+    cluster_barrier();
+    here = lane_id() >= c || *reinterpret_cast<volatile unsigned int*>(&ss.ended[lane_id()]) >= no;
+  } while (!__syncthreads_and(here));
+  return *reinterpret_cast<volatile unsigned int*>(&ss.failed) == 0u;
+}
+
 // The leader's part of a run of small levels, from level t.L (variant v, which
 // the log records) until the frontier outgrows the leader, the tree asks for a
 // pull, or nothing is left. ss.out holds the state before the run's first
 // level, and on return the state before the next level, whose frontier is in
-// the global queue (q[L & 1]) for the whole grid. (Not inlined: the kernel's
+// the global queue (q[L & 1]) for the whole grid. A run that a block's wait
+// failed in fails in every block. (Not inlined: the kernel's
 // other levels keep their registers. ubuf, sbuf, log and ss are in shared
 // memory.)
 template <int W>
@@ -318,6 +348,7 @@ __device__ __noinline__ void small_run(const DevGraph& g, const Buffers& b, uint
     ss.cnt[0] = ss.cnt[1] = ss.cnt[2] = 0u;
     ss.valid = ss.valid_won = ~0u;
     ss.leave = 0u;
+    ++ss.run_no;
   }
   __syncthreads();
   // the frontier from the global queue, vertex i to block i % c
@@ -396,13 +427,13 @@ __device__ __noinline__ void small_run(const DevGraph& g, const Buffers& b, uint
     const unsigned int count = min(ss.cnt[k3] & 0xffffu, ss.valid_won);
     for (unsigned int i = (unsigned)tid; i < count; i += kThreads) queue_append(qout, &st->small_tail, wonq[i]);
   }
+  ok = small_end(ss, c, rank, ss.run_no, ok);
   t.ok = ok ? 1 : 0;
   if (tid == 0) ss.out = t;
-  cluster_barrier();
   if (rank == 0u && tid == 0) {
     if (!ok) st->status = ST_TIMEOUT;
     st->small_tail = 0;
-    if (gridDim.x > c) {
+    if (gridDim.x > c && ss.mute == 0u) {
       st->small_out = t;
       __threadfence();
       st_release_u32(&st->small_seq, st->small_seq + 1u);
