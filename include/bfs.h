@@ -353,7 +353,7 @@ int bfs_batch_tune_ex(bfs_graph_t g, const int32_t* roots, int32_t k, int32_t* d
  * validated on every call (BFS_ERR_BAD_GRAPH). Synchronous: ordinary launches
  * (none cooperative, so the call runs beside other kernels on whatever part of
  * the GPU they leave free), the status read back after the first 8 to 20 levels
- * and then each time half as many again have run. Every level is the
+ * and then each time as many more have run (64 at most). Every level is the
  * edge-centric push (no tree switching).
  */
 int bfs_run_static(const int32_t* row_offsets, const int32_t* col_indices, int64_t n, int64_t m, int32_t root,

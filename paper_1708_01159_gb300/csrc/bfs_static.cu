@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kThreads, 4)
 // level past the last 1.7 us (3.3 with the vertices set aside). First what a
 // random graph of this mean degree needs, 1.75 ln n / ln(m / n) (6 levels for
 // R-MAT 14 and 18, 10 for Erdos-Renyi of 2^17 vertices and degree 8, 17 for 2^20
-// and 4), from then on half as many as have run.
+// and 4), from then on as many as have run.
 constexpr int32_t kFewestLevels = 8, kMostAtFirst = 20, kMostLevels = 64;
 int32_t levels_at_first(int64_t n, int64_t m) {
   const double degree = (double)m / (double)n;
@@ -239,7 +239,7 @@ int bfs_run_static(const int32_t* row_offsets, const int32_t* col_indices, int64
   TRY_LAUNCH("init");
   bool has_heavy = m >= kHeavy;  // as far as is known before the first read
   int32_t L = 0;
-  for (int32_t levels = levels_at_first(n, m); L <= nn; levels = std::min(std::max(L / 2, kFewestLevels), kMostLevels)) {
+  for (int32_t levels = levels_at_first(n, m); L <= nn; levels = std::min(std::max(L, kFewestLevels), kMostLevels)) {
     for (const int32_t end = L + levels; L < end; ++L) {
       cudaLaunchKernelEx(&cfg, k_static_level<false>, s, row_offsets, col_indices, depth_out, L);
       TRY_LAUNCH("level");
