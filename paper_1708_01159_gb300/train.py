@@ -16,8 +16,8 @@
               relative to the per-level optimum (the shape of Table 2).
   cv       -- k-fold cross-validation by graph over feature sets, weightings
               and depths.
-  holdout  -- each generator family (R-MAT, directed R-MAT, grid, ER) held out
-              in turn: trained on the others, evaluated on it (Section 4.4).
+  holdout  -- each generator family (R-MAT, directed R-MAT, grid, ER and the
+              other shapes) held out in turn: trained on the others, evaluated on it (Section 4.4).
   level-split -- the paper's random 70/30 split over levels: held-out
               per-level accuracy, for comparison with its reported accuracy.
 
@@ -188,11 +188,240 @@ TRAIN_GRAPHS = [
     ("rmat", dict(scale=12, edge_factor=24, seed=3113, permute=True)),
     ("rmat", dict(scale=11, edge_factor=32, seed=3114)),
     ("rmat", dict(scale=11, edge_factor=32, seed=3115, permute=True)),
+    # other shapes: a tree trained on R-MAT, grids and Erdos-Renyi alone pulled on
+    # stars (114 times the time of its predecessor's push) and on chains of cliques
+    ("smallworld", dict(n=4096, k=8, beta=0.1, seed=3116)),
+    ("smallworld", dict(n=16384, k=6, beta=0.01, seed=3117)),
+    ("smallworld", dict(n=30000, k=10, beta=0.1, seed=3118)),
+    ("smallworld", dict(n=131072, k=5, beta=0.05, seed=3119)),
+    ("smallworld", dict(n=524288, k=8, beta=0.2, seed=3120)),
+    ("smallworld", dict(n=1000000, k=6, beta=0.3, seed=3121)),
+    ("smallworld", dict(n=2097152, k=5, beta=0.02, seed=3122)),
+    ("growing", dict(n=8192, k=4, seed=3123)),
+    ("growing", dict(n=32768, k=8, seed=3124)),
+    ("growing", dict(n=262144, k=6, seed=3125)),
+    ("growing", dict(n=1048576, k=8, seed=3126)),
+    ("growing", dict(n=2097152, k=5, seed=3127)),
+    ("powerlaw", dict(n=8192, degree=8, exponent=2.3, seed=3128)),
+    ("powerlaw", dict(n=65536, degree=12, exponent=2.4, seed=3129)),
+    ("powerlaw", dict(n=262144, degree=8, exponent=2.2, seed=3130)),
+    ("powerlaw", dict(n=524288, degree=24, exponent=2.6, seed=3131)),
+    ("powerlaw", dict(n=1048576, degree=16, exponent=2.8, seed=3132)),
+    ("powerlaw", dict(n=2097152, degree=8, exponent=2.1, seed=3133)),
+    ("powerlaw", dict(n=32768, degree=8, exponent=2.3, seed=3134, directed=True)),
+    ("powerlaw", dict(n=262144, degree=16, exponent=2.4, seed=3135, directed=True)),
+    ("powerlaw", dict(n=1048576, degree=8, exponent=2.2, seed=3136, directed=True)),
+    ("moves", dict(dims=(200, 200), radius=1, seed=3137)),
+    ("moves", dict(dims=(400, 400), radius=2, seed=3138)),
+    ("moves", dict(dims=(700, 700), radius=2, seed=3139)),
+    ("moves", dict(dims=(250, 250), radius=3, seed=3140)),
+    ("moves", dict(dims=(128, 128), radius=4, seed=3141)),
+    ("moves", dict(dims=(1500, 200), radius=2, seed=3142)),
+    ("moves", dict(dims=(30, 30, 30), radius=1, seed=3143)),
+    ("moves", dict(dims=(90, 90, 90), radius=1, seed=3144)),
+    ("moves", dict(dims=(200, 60, 60), radius=1, seed=3145)),
+    ("moves", dict(dims=(50000,), radius=100, seed=3146)),
+    ("cliques", dict(count=300, size=16, seed=3147)),
+    ("cliques", dict(count=300, size=64, seed=3148)),
+    ("cliques", dict(count=100, size=200, seed=3149)),
+    ("cliques", dict(count=300, size=10, seed=3150)),
+    ("cliques", dict(count=60, size=400, seed=3151)),
+    ("cliques", dict(count=20, size=1000, seed=3152)),
+    ("stars", dict(n=3000, hubs=1, seed=3153)),
+    ("stars", dict(n=200000, hubs=1, seed=3154)),
+    ("stars", dict(n=500000, hubs=20, seed=3155)),
+    ("stars", dict(n=2000000, hubs=1000, seed=3156)),
+    ("stars", dict(n=100000, hubs=300, seed=3157)),
+    ("stars", dict(n=50000, hubs=3, seed=3158)),
+    ("stars", dict(n=20000, hubs=10, links=2, seed=3159)),
+    ("stars", dict(n=400000, hubs=50, links=2, seed=3160)),
+    ("stars", dict(n=1000000, hubs=2000, links=2, seed=3161)),
+    ("layers", dict(count=30, width=5000, k=8, seed=3162, directed=True)),
+    ("layers", dict(count=200, width=3000, k=12, seed=3163, directed=True)),
+    ("layers", dict(count=8, width=100000, k=16, seed=3164, directed=True)),
+    ("layers", dict(count=100, width=400, k=10, seed=3165, directed=True)),
+    ("layers", dict(count=20, width=100000, k=9, seed=3166, directed=True)),
+    ("layers", dict(count=300, width=20000, k=10, seed=3167)),
+    ("layers", dict(count=60, width=1000, k=20, seed=3168)),
+    ("bipartite", dict(left=300, right=3000, edges=50000, seed=3169)),
+    ("bipartite", dict(left=500, right=200000, edges=2000000, seed=3170)),
+    ("bipartite", dict(left=50000, right=50000, edges=1000000, seed=3171)),
+    ("bipartite", dict(left=5000, right=500000, edges=4000000, seed=3172)),
+    ("bipartite", dict(left=20, right=100000, edges=300000, seed=3173)),
+    ("regular", dict(n=65536, k=12, seed=3174)),
+    ("regular", dict(n=262144, k=10, seed=3175)),
+    ("regular", dict(n=1048576, k=16, seed=3176)),
+    ("regular", dict(n=3000, k=200, seed=3177)),
+    ("regular", dict(n=20000, k=64, seed=3178)),
+    ("rmat", dict(scale=14, edge_factor=16, a=0.45, b=0.22, c=0.22, seed=3179)),
+    ("rmat", dict(scale=17, edge_factor=8, a=0.45, b=0.22, c=0.22, seed=3180)),
+    ("rmat", dict(scale=21, edge_factor=12, a=0.45, b=0.22, c=0.22, seed=3181)),
+    ("rmat", dict(scale=16, edge_factor=16, a=0.7, b=0.1, c=0.1, seed=3182)),
+    ("rmat", dict(scale=19, edge_factor=16, a=0.7, b=0.1, c=0.1, seed=3183)),
+    ("rmat", dict(scale=20, edge_factor=2, seed=3184)),
+    ("rmat", dict(scale=22, edge_factor=4, seed=3185)),
+    ("rmat", dict(scale=17, edge_factor=8, a=0.45, b=0.22, c=0.22, seed=3186, directed=True)),
+    ("er", dict(n=262144, avg_degree=1.5, seed=3187)),
+    ("er", dict(n=2000, avg_degree=100.0, seed=3188)),
+    ("stars", dict(n=10000, hubs=2, seed=3189)),
+    ("stars", dict(n=30000, hubs=30, seed=3190)),
+    ("stars", dict(n=150000, hubs=5, seed=3191)),
+    ("stars", dict(n=300000, hubs=100, seed=3192)),
+    ("stars", dict(n=1500000, hubs=150, seed=3193)),
+    ("stars", dict(n=4000, hubs=4, links=2, seed=3194)),
+    ("stars", dict(n=60000, hubs=6, links=3, seed=3195)),
+    ("stars", dict(n=100000, hubs=40, links=2, seed=3196)),
+    ("stars", dict(n=200000, hubs=10, links=4, seed=3197)),
+    ("stars", dict(n=800000, hubs=20, links=2, seed=3198)),
+    ("stars", dict(n=1200000, hubs=200, links=3, seed=3199)),
+    ("tree", dict(n=100000, arity=10, seed=3200)),
+    ("tree", dict(n=1000000, arity=30, seed=3201)),
+    ("tree", dict(n=500000, arity=100, seed=3202)),
+    ("tree", dict(n=200000, arity=1000, seed=3203)),
+    ("tree", dict(n=1000000, arity=500, seed=3204)),
+    ("tree", dict(n=30000, arity=50, seed=3205)),
+    ("growing", dict(n=100000, k=1, seed=3206)),
+    ("growing", dict(n=1500000, k=1, seed=3207)),
+    ("growing", dict(n=400000, k=2, seed=3208)),
+    ("growing", dict(n=3000000, k=3, seed=3209)),
+    ("growing", dict(n=500000, k=16, seed=3210)),
+    ("hubs", dict(n=20000, degree=4, hubs=2, share=0.5, seed=3211)),
+    ("hubs", dict(n=100000, degree=3, hubs=10, share=0.2, seed=3212)),
+    ("hubs", dict(n=400000, degree=8, hubs=5, share=0.05, seed=3213)),
+    ("hubs", dict(n=1000000, degree=2, hubs=50, share=0.02, seed=3214)),
+    ("hubs", dict(n=1000000, degree=6, hubs=1, share=0.9, seed=3215)),
+    ("hubs", dict(n=200000, degree=1, hubs=30, share=0.03, seed=3216)),
+    ("components", dict(count=500, size=100, degree=10, seed=3217)),
+    ("components", dict(count=20, size=10000, degree=12, seed=3218)),
+    ("components", dict(count=4, size=300000, degree=10, seed=3219)),
+    ("components", dict(count=3000, size=400, degree=20, seed=3220)),
+    ("cliques", dict(count=150, size=100, seed=3221)),
+    ("cliques", dict(count=8, size=2000, seed=3222)),
+    ("cliques", dict(count=400, size=30, seed=3223)),
+    ("bipartite", dict(left=100, right=1000000, edges=3000000, seed=3224)),
+    ("bipartite", dict(left=2000, right=100000, edges=500000, seed=3225)),
+    ("bipartite", dict(left=1000000, right=1000000, edges=8000000, seed=3226)),
+    ("layers", dict(count=12, width=300000, k=12, seed=3227)),
+    ("layers", dict(count=150, width=8000, k=9, seed=3228)),
+    ("rmat", dict(scale=21, edge_factor=3, seed=3229)),
+    ("rmat", dict(scale=23, edge_factor=8, seed=3230)),
+    ("rmat", dict(scale=18, edge_factor=2, seed=3231)),
+    # R-MAT on vertex counts that are no power of two
+    ("rmatcut", dict(n=5000, edge_factor=8, seed=3232)),
+    ("rmatcut", dict(n=5657, edge_factor=24, seed=3233)),
+    ("rmatcut", dict(n=9187, edge_factor=12, seed=3234)),
+    ("rmatcut", dict(n=10438, edge_factor=16, seed=3235, directed=True)),
+    ("rmatcut", dict(n=17221, edge_factor=4, seed=3236)),
+    ("rmatcut", dict(n=17221, edge_factor=8, seed=3237)),
+    ("rmatcut", dict(n=24000, edge_factor=16, seed=3238)),
+    ("rmatcut", dict(n=24000, edge_factor=6, seed=3239, directed=True)),
+    ("rmatcut", dict(n=45098, edge_factor=8, seed=3240, directed=True)),
+    ("rmatcut", dict(n=45098, edge_factor=24, seed=3241)),
+    ("rmatcut", dict(n=70000, edge_factor=4, seed=3242)),
+    ("rmatcut", dict(n=90000, edge_factor=12, seed=3243)),
+    ("rmatcut", dict(n=100003, edge_factor=6, seed=3244, directed=True)),
+    ("rmatcut", dict(n=182362, edge_factor=16, seed=3245, directed=True)),
+    ("rmatcut", dict(n=182362, edge_factor=4, seed=3246)),
+    ("rmatcut", dict(n=300000, edge_factor=8, seed=3247)),
+    ("rmatcut", dict(n=300000, edge_factor=3, seed=3248)),
+    ("rmatcut", dict(n=419000, edge_factor=16, seed=3249)),
+    ("rmatcut", dict(n=419000, edge_factor=8, seed=3250, directed=True)),
+    ("rmatcut", dict(n=700000, edge_factor=4, seed=3251)),
+    ("rmatcut", dict(n=700000, edge_factor=12, seed=3252, directed=True)),
+    ("rmatcut", dict(n=1000003, edge_factor=8, seed=3253, directed=True)),
+    ("rmatcut", dict(n=1100000, edge_factor=12, seed=3254)),
+    ("rmatcut", dict(n=1234844, edge_factor=3, seed=3255)),
+    ("rmatcut", dict(n=1472023, edge_factor=16, seed=3256)),
+    ("rmatcut", dict(n=1472023, edge_factor=6, seed=3257, directed=True)),
+    ("rmatcut", dict(n=2500000, edge_factor=4, seed=3258)),
+    ("rmatcut", dict(n=2500000, edge_factor=8, seed=3259, directed=True)),
+    ("rmatcut", dict(n=3000000, edge_factor=12, seed=3260)),
+    ("rmatcut", dict(n=3500000, edge_factor=2, seed=3261)),
+    ("rmatcut", dict(n=3500000, edge_factor=16, seed=3262)),
+    ("er", dict(n=9742, avg_degree=4.0, seed=3263)),
+    ("er", dict(n=16384, avg_degree=4.0, seed=3264)),
+    ("er", dict(n=32768, avg_degree=4.0, seed=3265)),
+    ("er", dict(n=76173, avg_degree=4.0, seed=3266)),
+    ("er", dict(n=382885, avg_degree=4.0, seed=3267)),
+    ("er", dict(n=3000000, avg_degree=16.0, seed=3268)),
+    ("er", dict(n=2300000, avg_degree=12.0, seed=3269)),
+    ("er", dict(n=600000, avg_degree=6.0, seed=3270)),
 ]
 
 
+def shape_edges(kind, kw, rng):
+    """(vertices, sources, targets) of the generated shapes beside R-MAT, grids and
+    Erdos-Renyi: rings with rewired edges, preferential attachment, power-law
+    degrees, lattices whose moves reach every cell within a radius, chains of
+    cliques, stars (every leaf names `links` hubs in turn), trees, sparse random graphs
+    with hubs that name a share of all vertices, separate random components, layers
+    whose vertices name k of the next layer, random bipartite and regular graphs."""
+    if kind == "smallworld":
+        n, k = kw["n"], kw["k"]
+        s = np.repeat(np.arange(n), k)
+        t = (s + np.tile(np.arange(1, k + 1), n)) % n
+        moved = rng.random(n * k) < kw["beta"]
+        return n, s, np.where(moved, rng.integers(0, n, n * k), t)
+    if kind == "growing":
+        n, k = kw["n"], kw["k"]
+        s = np.repeat(np.arange(n), k)
+        return n, s, (rng.random(n * k) ** 2 * s).astype(np.int64)
+    if kind == "powerlaw":
+        n, m = kw["n"], kw["n"] * kw["degree"] // (1 if kw.get("directed") else 2)
+        c = np.cumsum(np.arange(1, n + 1) ** (-1.0 / (kw["exponent"] - 1.0)))
+        return n, np.searchsorted(c, rng.random(m) * c[-1]), np.searchsorted(c, rng.random(m) * c[-1])
+    if kind == "moves":
+        dims, r = kw["dims"], kw["radius"]
+        n = int(np.prod(dims))
+        at = np.unravel_index(np.arange(n), dims)
+        src, dst = [], []
+        for move in np.ndindex(*([2 * r + 1] * len(dims))):
+            d = np.array(move) - r
+            if tuple(d) <= (0,) * len(dims):
+                continue
+            to = [x + int(y) for x, y in zip(at, d)]
+            ok = np.logical_and.reduce([(x >= 0) & (x < e) for x, e in zip(to, dims)])
+            src.append(np.nonzero(ok)[0])
+            dst.append(np.ravel_multi_index([x[ok] for x in to], dims))
+        return n, np.concatenate(src), np.concatenate(dst)
+    if kind == "cliques":
+        n, c = kw["count"] * kw["size"], kw["size"]
+        i = np.arange(n)
+        pairs = [(i[i % c + j < c], i[i % c + j < c] + j) for j in range(1, c)]
+        pairs.append((i[:-1][i[:-1] % c == c - 1], i[1:][i[:-1] % c == c - 1]))
+        return n, np.concatenate([p[0] for p in pairs]), np.concatenate([p[1] for p in pairs])
+    if kind == "stars":
+        n, h = kw["n"], kw["hubs"]
+        leaves = np.arange(h, n)
+        s = np.repeat(leaves, kw.get("links", 1))
+        t = (s + np.tile(np.arange(kw.get("links", 1)), n - h)) % h
+        return n, s, t
+    if kind == "tree":
+        child = np.arange(1, kw["n"])
+        return kw["n"], child, (child - 1) // kw["arity"]
+    if kind == "hubs":
+        n, m, h = kw["n"], kw["n"] * kw["degree"] // 2, int(kw["n"] * kw["share"])
+        s = np.concatenate([rng.integers(0, n, m), np.repeat(np.arange(kw["hubs"]), h)])
+        return n, s, rng.integers(0, n, len(s))
+    if kind == "components":
+        n, c = kw["count"] * kw["size"], kw["size"]
+        s = rng.integers(0, n, n * kw["degree"] // 2)
+        return n, s, s // c * c + rng.integers(0, c, len(s))
+    if kind == "layers":
+        w, k = kw["width"], kw["k"]
+        s = np.repeat(np.arange((kw["count"] - 1) * w), k)
+        return kw["count"] * w, s, (s // w + 1) * w + rng.integers(0, w, len(s))
+    if kind == "bipartite":
+        n = kw["left"] + kw["right"]
+        return n, rng.integers(0, kw["left"], kw["edges"]), kw["left"] + rng.integers(0, kw["right"], kw["edges"])
+    if kind == "regular":
+        n, k = kw["n"], kw["k"]
+        return n, np.tile(np.arange(n), k // 2), np.concatenate([rng.permutation(n) for _ in range(k // 2)])
+    raise ValueError(kind)
+
+
 def family(name: str) -> str:
-    """Generator family of a training graph's name: rmat, rmat-dir, grid or er."""
+    """Generator family of a training graph's name: rmat, rmat-dir, grid, er or another shape's kind."""
     if name.startswith("rmat"):
         return "rmat-dir" if name.endswith("-dir") else "rmat"
     return name.split("-")[0]
@@ -207,7 +436,19 @@ def make_graph(kind, kw):
         return gg.grid(kw["rows"], kw["cols"], kw["drop"], seed=kw["seed"], permute=True)
     if kind == "er":
         return gg.erdos_renyi(kw["n"], kw["avg_degree"], seed=kw["seed"])
-    raise ValueError(kind)
+    directed = bool(kw.get("directed"))
+    if kind == "rmatcut":  # R-MAT over the next power of two, its first n ids
+        n = kw["n"]
+        g = gg.rmat((n - 1).bit_length(), kw["edge_factor"], seed=kw["seed"], directed=directed)
+        s, t = np.repeat(np.arange(g.n), np.diff(g.off)), g.idx
+        ok = (s < n) & (t < n)
+        return gg.from_edges(n, s[ok], t[ok], symmetrize=not directed,
+                             name=f"rmatcut-n{n}-seed{kw['seed']}" + ("-dir" if directed else ""))
+    rng = np.random.default_rng(kw["seed"])
+    n, s, t = shape_edges(kind, kw, rng)
+    p = rng.permutation(n)  # ids in random order
+    return gg.from_edges(n, p[s], p[t], symmetrize=not directed,
+                         name=f"{kind}-n{n}-seed{kw['seed']}" + ("-dir" if directed else ""))
 
 
 def collect(out: str, roots_per_graph: int = 4, reps: int = 3, max_levels: int = 16384, graphs=None):
@@ -284,7 +525,8 @@ def level_weights(T, trav, weighting):
     slowdown that Table 2 averages. 'cost': as 'relregret', with the spread cut
     at four times the level's best (one whole-graph pull of a hub's list costs a
     thousand levels) and half the step to the second best added, so that close
-    calls count too; its leaves are labelled by cost (fit)."""
+    calls count too; its tree is pruned and its leaves are labelled by the full
+    costs (fit)."""
     if weighting == "uniform":
         return np.ones(len(T))
     spread = T.max(axis=1) - T.min(axis=1) + 1e-5
@@ -307,51 +549,108 @@ def traversal_optimum(T, trav):
 
 # The library evaluates trees of up to 64 leaves in their bit-parallel form,
 # held in shared memory (larger ones are walked node by node in global
-# memory, about 1 us per level); the exporter keeps to that.
+# memory, about 1 us per level); the exporter keeps to that. (What counts is the
+# tree left once a graph's own tests are decided; but of 192 leaves that rest had
+# 36 where 64 leave 20, and its evaluation cost 1 to 2.5 % of small traversals.)
 MAX_LEAVES = 64
+GROWN_LEAVES = 1000  # of a tree that is pruned
 
 
 def fit(X, T, feature_idx, max_depth=8, min_samples_leaf=8, weighting="regret", trav=None, max_leaves=MAX_LEAVES):
     """CART with Gini impurity (Section 2.1); labels: the fastest variant per level.
-    Under the 'cost' weighting each leaf is labelled with the variant of least
-    total time over its levels (each level's times over its traversal's optimum)
-    instead of the heaviest class: clf.leaf_label_, by node."""
+    Under the 'cost' weighting the tree is grown larger and pruned back by cost
+    (prune), and each leaf is labelled with the variant of least total cost over its
+    levels (each level's times over its traversal's optimum) instead of the heaviest
+    class: clf.leaf_label_, by node."""
     from sklearn.tree import DecisionTreeClassifier
     y = T.argmin(axis=1)
     w = level_weights(T, trav if trav is not None else np.zeros(len(T)), weighting)
+    grown = max(GROWN_LEAVES, max_leaves) if weighting == "cost" else max_leaves
     clf = DecisionTreeClassifier(criterion="gini", max_depth=max_depth, min_samples_leaf=min_samples_leaf,
-                                 max_leaf_nodes=max_leaves, random_state=0)
+                                 max_leaf_nodes=grown, random_state=0)
     clf.fit(X[:, feature_idx], y, sample_weight=w)
     if weighting == "cost":
-        cost = T / traversal_optimum(T, trav)[:, None]
-        leaf = clf.apply(X[:, feature_idx].astype(np.float32))
-        clf.leaf_label_ = {int(k): int(cost[leaf == k].sum(axis=0).argmin()) for k in np.unique(leaf)}
+        cost = np.zeros((clf.tree_.node_count, T.shape[1]))
+        np.add.at(cost, clf.apply(X[:, feature_idx].astype(np.float32)), T / traversal_optimum(T, trav)[:, None])
+        prune(clf, cost, max_leaves)
     return clf
+
+
+def prune(clf, cost, max_leaves):
+    """Cost-complexity pruning (Breiman et al. 1984) with the levels' cost in place of
+    the misclassification rate: while there are too many leaves, the subtree whose
+    leaves save the least cost each over its root as a leaf is cut. cost: by leaf and
+    variant. Sets clf.leaf_label_ (the variant of least cost of every leaf left)."""
+    left, right = clf.tree_.children_left, clf.tree_.children_right
+    order, todo = [], [0]
+    while todo:
+        i = todo.pop()
+        order.append(i)
+        if left[i] >= 0:
+            todo += [left[i], right[i]]
+    parent = np.full(len(left), -1)
+    leaves = np.ones(len(left), dtype=np.int64)
+    for i in reversed(order):
+        if left[i] >= 0:
+            cost[i] = cost[left[i]] + cost[right[i]]
+            parent[left[i]] = parent[right[i]] = i
+    own = cost.min(axis=1)
+    sub = own.copy()
+    for i in reversed(order):
+        if left[i] >= 0:
+            sub[i] = sub[left[i]] + sub[right[i]]
+            leaves[i] = leaves[left[i]] + leaves[right[i]]
+    inner = {i for i in order if left[i] >= 0}
+    while leaves[0] > max_leaves:
+        cut = min(inner, key=lambda i: ((own[i] - sub[i]) / (leaves[i] - 1), i))
+        up, gain, gone = parent[cut], own[cut] - sub[cut], leaves[cut] - 1
+        todo = [cut]
+        while todo:
+            i = todo.pop()
+            if i in inner:
+                inner.discard(i)
+                todo += [left[i], right[i]]
+        sub[cut], leaves[cut] = own[cut], 1
+        while up >= 0:
+            sub[up] += gain
+            leaves[up] -= gone
+            up = parent[up]
+    kept = [i for i in order if i == 0 or parent[i] in inner]
+    clf.leaf_label_ = {int(i): int(cost[i].argmin()) for i in kept if i not in inner}
 
 
 def export(clf, feature_idx, path, meta=""):
     """Integer tree text: 'feature threshold left right value' per node."""
     t = clf.tree_
+    labels = getattr(clf, "leaf_label_", None)
+    nodes, todo = [], [0]  # what is left of a pruned tree
+    while todo:
+        i = todo.pop()
+        nodes.append(i)
+        if t.children_left[i] >= 0 and not (labels and i in labels):
+            todo += [t.children_left[i], t.children_right[i]]
+    nodes.sort()  # a parent before its children
+    number = {i: k for k, i in enumerate(nodes)}
     lines = []
-    for i in range(t.node_count):
-        if t.children_left[i] < 0:
+    for i in nodes:
+        if t.children_left[i] < 0 or (labels and i in labels):
             v = t.value[i][0]
             order = np.argsort(v)[::-1]
             cls = clf.classes_
             top = int(cls[order[0]])
             tie = len(order) > 1 and math.isclose(float(v[order[0]]), float(v[order[1]]), rel_tol=1e-9)
-            labels = getattr(clf, "leaf_label_", None)
             lines.append(f"-1 0 -1 -1 {labels[i] if labels else -1 if tie else top}")
         else:
             f = int(feature_idx[t.feature[i]])
-            lines.append(f"{f} {int(math.floor(t.threshold[i]))} {t.children_left[i]} {t.children_right[i]} -1")
+            lines.append(f"{f} {int(math.floor(t.threshold[i]))} {number[t.children_left[i]]} "
+                         f"{number[t.children_right[i]]} -1")
     with open(path, "w") as fh:
         fh.write("# Decision tree trained on per-level GB300 timings (CART, Gini).\n")
         for m in meta.splitlines():
             fh.write(f"# {m}\n")
         fh.write("# Features: " + ", ".join(f"{i} {f}" for i, f in enumerate(FEATURES)) + "\n")
         fh.write("# Classes: " + ", ".join(f"{i} {v}" for i, v in enumerate(VARIANTS)) + "\n")
-        fh.write(f"bfs-tree 1 {t.node_count}\n")
+        fh.write(f"bfs-tree 1 {len(nodes)}\n")
         fh.write("\n".join(lines) + "\n")
 
 
