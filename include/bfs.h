@@ -297,7 +297,8 @@ typedef struct bfs_batch_config {
   int32_t grid_blocks; /* blocks of the multi-source kernel (larger values are clamped to one full
                           occupancy wave); 0 for a grid sized to the graph: one block per 1024
                           vertices, at least a quarter of the SMs, at most one full occupancy
-                          wave (so that small graphs' waves on several streams run together) */
+                          wave (so that small graphs' waves on several streams run together),
+                          and fewer for large graphs without in-lists of 192 entries or more */
 } bfs_batch_config;
 
 /* Set the graph's multi-source configuration. Errors: BFS_ERR_INVALID_ARG. */

@@ -868,6 +868,32 @@ int ms_prepare(bfs_graph* g) {
 
 // One wave of up to 64 roots (host array) into the k output rows (host array
 // of device pointers) on the given set.
+// Blocks of a wave of k roots when the caller names none: at least a quarter of
+// the SMs, at most one full occupancy wave, and in between sized to the graph, so
+// that waves of small graphs on different streams can be resident together and a
+// level's barriers do not wait for more blocks than have work.
+//  - Lists long enough to be dealt over the grid: a block per 1024 vertices (ten
+//    R-MAT graphs of 4,096 to 262,144 vertices on five streams: 1.43 ms with a
+//    block per 4096 vertices, 0.94 per 2048, 0.76 per 1024, 0.89 per 512).
+//  - Others: the same up to two blocks an SM, a block per 2304 vertices past that
+//    (Erdos-Renyi 2^20 of degree 8, 64 roots: 606 us on 760 blocks, 531 on 456, 572
+//    on 304; 2^19: 412, 326, 318).
+//  - Out-degrees of at most 8, where levels may be many and small: up to one block
+//    an SM, two for 32 roots or more, a block per 4096 vertices past that (1000 x
+//    1000 grid: one root 38.4 ms on 760 blocks, 19.8 on 304, 16.5 on 152; 64 roots
+//    72, 47, 51; 2^18 vertices of out-degree 8: one root 160 us on 256 blocks, 158
+//    on 152, 64 roots 206 and 226).
+int ms_default_grid(const bfs_graph* g, int32_t k) {
+  const long long n = g->dg.n, sms = std::max(1, g->sms);
+  const auto per = [n](long long vertices) { return (n + vertices - 1) / vertices; };
+  long long blocks = per(1024);
+  if (g->dg.gfeat[F_IN_DEG_MAX] < kMsLongList) {
+    const bool low = g->dg.gfeat[F_DEG_MAX] <= 8;
+    blocks = std::max(std::min(blocks, low && k < 32 ? sms : 2 * sms), per(low ? 4096 : 2304));
+  }
+  return (int)std::min<long long>(std::max(blocks, std::max(1ll, sms / 4)), g->ms_grid);
+}
+
 int ms_launch_wave(bfs_graph* g, MsSet* set, const int32_t* roots, int32_t k, int32_t* const* rows_out,
                    cudaStream_t s, MsConfig cfg, int32_t grid_blocks = 0) {
   MsRows rows{};
@@ -882,13 +908,7 @@ int ms_launch_wave(bfs_graph* g, MsSet* set, const int32_t* roots, int32_t k, in
   MsState* st = set->st;
   int32_t stall = take_stall();
   void* args[] = {&dg, &mb, &st, &k, &rows, &cfg, &stall};
-  // default: a grid sized to the graph (one block per 1024 vertices, at least
-  // a quarter of the SMs, at most one full occupancy wave), so that waves of
-  // small graphs on different streams can be resident together. Ten R-MAT
-  // graphs of 4,096 to 262,144 vertices on five streams: 1.43 ms with a block
-  // per 4096 vertices, 0.94 per 2048, 0.76 per 1024, 0.89 per 512.
-  const long long sized = std::max<long long>(((long long)g->dg.n + 1023) / 1024, std::max(1, g->sms / 4));
-  const int grid = grid_blocks > 0 ? std::min(grid_blocks, g->ms_grid) : (int)std::min<long long>(sized, g->ms_grid);
+  const int grid = grid_blocks > 0 ? std::min(grid_blocks, g->ms_grid) : ms_default_grid(g, k);
   CU(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_msbfs), dim3(grid), dim3(kMsThreads), args, 0, s));
   return BFS_OK;
 }

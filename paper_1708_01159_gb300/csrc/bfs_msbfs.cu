@@ -59,9 +59,7 @@ namespace {
 
 constexpr unsigned kFullMask = 0xffffffffu;
 constexpr int kMsTile = kMsThreads;      // push_mode 0: frontier vertices whose edges a block deals out together
-constexpr int kMsRounds = 16;            // pull: rounds of four in-neighbours a lane looks at for its own vertex
-constexpr int32_t kMsLong = 128;         // pull: in-neighbours left from which all blocks look at them together
-constexpr int32_t kMsChunk = 128;        // of which a warp takes so many at a time
+constexpr int32_t kMsChunk = 128;        // pull, a list dealt over the grid: entries a warp takes at a time
 
 // Predicated accesses, one instruction each (see ld_if in bfs_internal.cuh).
 __device__ __forceinline__ unsigned long long ld64_if(bool p, const unsigned long long* a, unsigned long long otherwise) {
@@ -215,7 +213,7 @@ __global__ void __launch_bounds__(kMsThreads, 5) k_msbfs(DevGraph g, MsBuffers m
   }
   bool ok = grid_arrive_wait(&st->bar64, bar_target, &st->status);
   const int64_t words = (n + 31) / 32;
-  const bool has_long = g.gfeat[F_IN_DEG_MAX] >= kMsLong + 4 * kMsRounds;  // some pull may set a vertex aside
+  const bool has_long = g.gfeat[F_IN_DEG_MAX] >= kMsLongList;  // some pull may set a vertex aside
   int32_t L = 0;
   for (; ok; ++L) {
     const unsigned int f = *reinterpret_cast<volatile unsigned int*>(&st->ftail[L % 4]);

@@ -7,6 +7,11 @@ namespace bfs {
 
 constexpr int kMsThreads = 256;
 constexpr int kMsMaxRoots = 64;
+// In-lists from this length on may be set aside by a pull level and dealt over the
+// grid: what a lane looks at itself, and what is worth dealing.
+constexpr int kMsRounds = 16;       // rounds of four in-neighbours a lane looks at for its own vertex
+constexpr int32_t kMsLong = 128;    // in-neighbours left from which all blocks look at them together
+constexpr int32_t kMsLongList = kMsLong + 4 * kMsRounds;
 // Depths below this value are recorded in the per-level history (one mask per
 // vertex and depth) until the wave ends; deeper ones are written to the output
 // when found.
