@@ -68,8 +68,6 @@ __device__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity) {
   return true;
 }
 
-
-
 __device__ __forceinline__ Level load_level(const DevGraph& g, const Buffers& b, RunState* st) {
   Level lv;
   // select with ternaries: indexing the by-value parameter arrays would copy them to local memory
@@ -1068,8 +1066,6 @@ __global__ void __launch_bounds__(kThreads) k_pull(DevGraph g, Buffers b, RunSta
 // ===========================================================================
 // Persistent path: the whole traversal in one cooperative launch
 // ===========================================================================
-// Clears the words the persistent kernel's blocks read before block 0 could
-// reset them (a previous run may have stopped with an error).
 // Timing harness: undo one level run from the graph path's state. The vertices
 // the level discovered are exactly the entries it appended to the output
 // queue, so resetting their depth and visited bit restores the state it
@@ -1087,7 +1083,6 @@ __global__ void k_undo_level(Buffers b, RunState* st) {
     atomicAnd(&vis[v >> 5], ~(1u << (v & 31)));
   }
 }
-
 
 // One shared-memory buffer serves the CTA variant's copy stage or the
 // edge-centric tile of the persistent kernels.
@@ -1210,6 +1205,9 @@ namespace bfs {
 // stall: STALL_NONE, or the test hook's choice of one bounded wait to run out.
 // kRecord: 0, or the entries of the graph's vertex records (4 or 8); then small
 // levels run on the leader cluster (bfs_small.cuh).
+// Four blocks an SM: at their 64 registers 60 to 68 bytes a thread are spilled (120
+// to 144 read back); five blocks at 48 registers spilled 216 and ran R-MAT 22 9 %
+// slower.
 template <int kRecord>
 __global__ void __launch_bounds__(kThreads, 4) k_bfs_persistent(const __grid_constant__ DevGraph g,
                                                              const __grid_constant__ Buffers b, RunState* st,

@@ -137,6 +137,7 @@ __device__ __forceinline__ void ms_record(const MsBuffers& mb, const MsRows& row
 
 }  // namespace
 
+// Five blocks an SM: 48 registers, 60 bytes a thread spilled (88 read back).
 __global__ void __launch_bounds__(kMsThreads, 5) k_msbfs(DevGraph g, MsBuffers mb, MsState* st, int32_t k,
                                                        MsRows rows, MsConfig cfg, int32_t stall) {
   __shared__ unsigned long long s_edges[64];

@@ -23,10 +23,12 @@
 // the rate at which 16 SMs issue scattered requests. 4096^2 grid with a tenth
 // of the edges dropped (6,194 levels, 2,708 vertices and 9,750 edges on
 // average): 6.66 us a level on the whole grid, 2.76 us here (1.9 below 1,024
-// vertices, 3.6 above 4,096), the traversal 41.3 -> 17.1 ms. Other forms
-// measured on the same graph: row extents and lists read from the CSR by four
-// edges of a thread 28.4 ms; records without the prefetch 23.8; 8 blocks
-// instead of 16 32.0; two candidates a thread at most instead of four 20.9.
+// vertices, 3.6 above 4,096), the traversal 41.3 -> 17.1 ms (17.1 to 20.2 over
+// boxes and roots). Other forms measured on the same graph and box: row extents
+// and lists read from the CSR by four edges of a thread 28.4 ms; records without
+// the prefetch 23.8; 8 blocks instead of 16 32.0; two candidates a thread at most
+// instead of four 20.9. At the 64 registers of the persistent kernel small_run<4>
+// spills 108 bytes on the way, in the graph driver's kernel (80 registers) none.
 #pragma once
 
 namespace bfs {
